@@ -133,8 +133,8 @@ typedef struct sparkling_proj {
 #define SPARKLING_KERNEL_COUNT 8
 
 /* Arithmetic of the projection (sparkling_set_projection). */
-#define SPARKLING_PROJECTION_FP64 0    /* duals, primal and step in FP64 for every K dtype (default) */
-#define SPARKLING_PROJECTION_MIXED 1   /* FP32 K, fixed n_iter: FP32 iteration on s - k and the duals */
+#define SPARKLING_PROJECTION_FP64 0    /* FP64, or 48-bit two-float sums where the result is FP32 (default) */
+#define SPARKLING_PROJECTION_MIXED 1   /* FP32 K, fixed n_iter: FP32 iteration allowed */
 
 /* How sparkling_step runs its device work (sparkling_set_step_path). */
 #define SPARKLING_STEP_AUTO 0      /* the persistent engine from 2^22 samples on, else the kernels (default) */
@@ -224,8 +224,8 @@ SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, i
 
 /* Projection of each of Nc shots of Ns samples onto the constraint set
  * (Sec. II-D, Suppl. Sec. I), in place on K ([Nc*Ns][3], K_dtype), with the
- * dual FISTA iteration in FP64 (sparkling_set_projection: the opt-in mixed
- * form for FP32 K):
+ * dual FISTA iteration in FP64 (or, for FP32 K, in two-float sums of 48 bits,
+ * see sparkling_set_projection):
  *   D1 s[n] = s[n+1]-s[n], D2 s[n] = s[n+2]-2s[n+1]+s[n];
  *   s(q) = pin(clip_box(k - D1^T q1 - D2^T q2)); step tau = 1/20;
  *   z = y + tau D s(y); q+ = z - P_ball(tau*alpha or tau*beta)(z) per row;
@@ -260,9 +260,11 @@ SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64
  * the packing of samples and densities): a work list of attraction items (a
  * tile of 1024 targets against a run of grid rows) and symmetric repulsion
  * items (a tile of targets against a run of source tiles, each unordered
- * pair once, exact fixed-point totals per sample), followed by one
- * projection item per shot that waits (bounded) for its trajectory's pair
- * items.  With SPARKLING_BATCH_TWO_LAUNCHES (and wherever the one-launch
+ * pair once, exact fixed-point totals per sample).  FP32 trajectories are
+ * then projected in a second launch (one CTA or cluster per shot, the form of
+ * sparkling_project); FP64 ones, and FP32 ones that form does not cover, by
+ * one projection item per shot of the same list, which waits (bounded) for
+ * its trajectory's pair items.  With SPARKLING_BATCH_TWO_LAUNCHES (and wherever the one-launch
  * kernel shape cannot be resident) the symmetric repulsion of every
  * trajectory runs first in its own kernel -- the same totals bit for bit --
  * and the persistent kernel's list holds only the attraction and projection
@@ -393,12 +395,16 @@ SPARKLING_API int sparkling_set_regularisation(sparkling_ctx *ctx, double eps);
 /* Arithmetic of the context's projections (sparkling_project, sparkling_step,
  * sparkling_step_host, sparkling_step_batched, the driver).
  *   SPARKLING_PROJECTION_FP64 (default): the dual FISTA iteration, the primal
- *     map and the step in FP64 for every K dtype; the result is rounded to
- *     K_dtype once.
- *   SPARKLING_PROJECTION_MIXED: for FP32 K with a fixed n_iter, the iteration
- *     runs in FP32 on the displacement e = s - k and the duals (D1 k, D2 k and
- *     the box and pin offsets formed once per shot in FP64, the output
- *     k + e in FP64); FP64 K and converged mode keep the FP64 iteration.
+ *     map and the step in FP64; the result is rounded to K_dtype once.  For
+ *     FP32 K with a fixed n_iter <= 4096, Ns <= 8192 and alpha, beta (or inf),
+ *     box and pin in [2^-40, 2^40], the duals and the primal map are carried
+ *     as unevaluated sums of two floats (48 bits; the step k = K - eta G in
+ *     FP64) -- the FP32 result is the FP64 one up to its last rounding.
+ *   SPARKLING_PROJECTION_MIXED: lets FP32 K with a fixed n_iter iterate in
+ *     FP32 on the displacement e = s - k and the duals (D1 k, D2 k and the box
+ *     and pin offsets formed once per shot in FP64, the output k + e in FP64)
+ *     where the two-float form does not apply (it is both faster and more
+ *     accurate); FP64 K and converged mode keep the FP64 iteration.
  * Returns SPARKLING_E_INVAL for another mode. */
 SPARKLING_API int sparkling_set_projection(sparkling_ctx *ctx, int mode);
 

@@ -331,8 +331,8 @@ def sparkling_step_batched(ctx: Context, K, traj_off: Sequence[int], Ns: int,
                            acc: int = ACC_KAHAN32, graph: bool = True, one_launch: bool = True,
                            stream=None):
     """One projected-gradient step of B trajectories (samples
-    [traj_off[b], traj_off[b+1]) of K), in place, in one persistent launch;
-    one_launch=False runs the symmetric repulsion in its own kernel first."""
+    [traj_off[b], traj_off[b+1]) of K), in place: one persistent launch of the
+    pair work, FP32 projections in a second one; one_launch=False runs the symmetric repulsion in its own kernel first."""
     B = len(grids)
     if len(traj_off) != B + 1 or len(etas) != B or len(projs) != B:
         raise ValueError("traj_off needs B+1 entries, etas and projs B")
@@ -406,8 +406,8 @@ def sparkling_set_attraction(ctx: Context, mode: int) -> None:
 
 
 def sparkling_set_projection(ctx: Context, mode: int) -> None:
-    """PROJECTION_FP64 (default: FP64 iteration for every K dtype) or
-    PROJECTION_MIXED (FP32 K: FP32 iteration on the displacement)."""
+    """PROJECTION_FP64 (default: FP64 iteration, or 48-bit two-float sums for
+    FP32 K) or PROJECTION_MIXED (FP32 K: an FP32 iteration is allowed)."""
     _check(ctx, lib().sparkling_set_projection(ctx.handle, int(mode)))
 
 

@@ -37,6 +37,7 @@ struct sparkling_ctx {
     int proj_mode = SPARKLING_PROJECTION_FP64;
     int step_path = SPARKLING_STEP_AUTO;
     double *d_small = nullptr;  // [0..1] energy, [2..5] violation bits, [6] notconv (int)
+    void *d_mom = nullptr;      // momentum factors of the projection (MomentumTables)
     void *ws = nullptr;
     size_t ws_bytes = 0;
     // host-buffer entry points keep their device copies here
@@ -80,6 +81,8 @@ struct sparkling_ctx {
         std::vector<EngineItem> items;
         std::vector<size_t> o_rho, o_coords;
         size_t o_pos = 0, o_traj = 0, o_items = 0, o_cnt = 0, o_part = 0, o_gstate = 0, end = 0;
+        bool split_proj = false;          // projections in a launch of their own
+        RegShape proj_shape;              // its shape
         bool sym = false;                 // repulsion by the batched symmetric kernel
         bool one_launch = false;          // symmetric repulsion items in the engine's work list
         bool roles = false;               // role dispatch over the list's three parts
@@ -158,6 +161,38 @@ int cuda_fail(sparkling_ctx *ctx, cudaError_t e, const char *what)
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call);                                   \
     } while (0)
 
+// FISTA momentum t+ = (1 + sqrt(1 + 4 t^2))/2, mom = (t - 1)/t+: (mom_it,
+// mom_{it+1}) as doubles, (1 + mom_it, mom_{it+1}) as two-float sums.
+int upload_momentum(sparkling_ctx *ctx)
+{
+    std::vector<double2> d(kMomentumMax);
+    std::vector<float4> f(kMomentumMax);
+    auto split = [](double v, float &h, float &l) { h = (float)v; l = (float)(v - (double)h); };
+    double t = 1.0, mom = 0.0;
+    for (int it = 0; it < kMomentumMax; ++it) {
+        d[it].x = mom;
+        split(1.0 + mom, f[it].x, f[it].y);
+        t = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
+        const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
+        mom = (t - 1.0) / tn;
+        d[it].y = mom;
+        split(d[it].y, f[it].z, f[it].w);
+    }
+    const size_t nd = d.size() * sizeof(double2), nf = f.size() * sizeof(float4);
+    CK(cudaMalloc(&ctx->d_mom, nd + nf));
+    CK(cudaMemcpy(ctx->d_mom, d.data(), nd, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(static_cast<char *>(ctx->d_mom) + nd, f.data(), nf, cudaMemcpyHostToDevice));
+    return SPARKLING_OK;
+}
+
+MomentumTables momentum_tables(const sparkling_ctx *ctx)
+{
+    MomentumTables m;
+    m.d = static_cast<const double2 *>(ctx->d_mom);
+    m.f = reinterpret_cast<const float4 *>(m.d + kMomentumMax);
+    return m;
+}
+
 int lazy_init(sparkling_ctx *ctx)
 {
     if (ctx->inited) {
@@ -176,6 +211,8 @@ int lazy_init(sparkling_ctx *ctx)
     CK(cudaMemcpy(ctx->d_status, &ctl, sizeof(DevCtl), cudaMemcpyHostToDevice));
     CK(cudaMalloc(&ctx->d_small, 8 * sizeof(double)));
     CK(cudaMemset(ctx->d_small, 0, 8 * sizeof(double)));
+    int s;
+    if ((s = upload_momentum(ctx))) return s;
     ctx->inited = true;
     return SPARKLING_OK;
 }
@@ -809,14 +846,21 @@ int common_checks(sparkling_ctx *ctx, const void *K, int K_dtype, int64_t N, con
 // Launch shape of the projection: one CTA per shot up to one wave; the
 // per-CTA state goes to the workspace when it does not fit in shared memory.
 struct ProjPlan {
+    RegShape reg;                // state in registers (ctas > 0), else as below
     int grid = 0;
     bool global_state = false;
     size_t o_state = 0;
 };
 
-int plan_project(sparkling_ctx *ctx, int K_dtype, int64_t Nc, int64_t Ns, Carve &cv, ProjPlan &L)
+int plan_project(sparkling_ctx *ctx, int K_dtype, int64_t Nc, int64_t Ns, const sparkling_proj *pr,
+                 Carve &cv, ProjPlan &L)
 {
     const int ns = (int)Ns;
+    if (project_reg_applies(K_dtype, ns, pr->alpha, pr->beta, pr->box, pr->tol, pr->pin,
+                            pr->pin_index, pr->n_iter)) {
+        L.reg = project_reg_shape(K_dtype, Nc, ns, ctx->sms);
+        return SPARKLING_OK;
+    }
     const int occ = project_ctas_per_sm(K_dtype, ns);
     if (occ < 1) {
         cudaGetLastError();
@@ -851,9 +895,13 @@ int run_project(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t Ns
     p.mixed = ctx->proj_mode == SPARKLING_PROJECTION_MIXED ? 1 : 0;
     if (want_viol || p.notconv)
         CK(cudaMemsetAsync(ctx->d_small + 2, 0, 5 * sizeof(double), st));
+    p.mom = momentum_tables(ctx);
     LaunchScope ls(ctx, SPARKLING_KERNEL_PROJECT, st);
-    CK(launch_project(p, K_dtype, L.grid, st));
-    ls.done();
+    if (L.reg.ctas > 0)
+        CK(launch_project_reg(p, K_dtype, L.reg, ctx->sms, st));
+    else
+        CK(launch_project(p, K_dtype, L.grid, st));
+    ls.done(L.reg.ctas > 0 && want_viol ? 2 : 1);
     return SPARKLING_OK;
 }
 
@@ -908,7 +956,7 @@ int64_t pair_cost(int64_t N, int64_t P) { return N * P + N * N; }
 // wait of a projection item end.
 void build_work_list(sparkling_ctx::Batch &b, const std::vector<int64_t> &off,
                      const sparkling_grid *grids, int ctas, int items_per_cta, bool sym,
-                     bool one_launch)
+                     bool one_launch, bool project)
 {
     const int B = (int)off.size() - 1;
     int64_t total = 0;
@@ -924,6 +972,7 @@ void build_work_list(sparkling_ctx::Batch &b, const std::vector<int64_t> &off,
     b.n_pair_items = 0;
     b.n_lead_items = -1;
     auto project_items = [&](int t) {
+        if (!project) return;
         if (b.n_lead_items < 0) b.n_lead_items = (int64_t)b.items.size();
         for (int c = 0; c < b.traj[t].Nc; ++c) {
             EngineItem it;
@@ -1012,6 +1061,7 @@ void build_work_list(sparkling_ctx::Batch &b, const std::vector<int64_t> &off,
             project_items(released++);
     }
     while (released < B) project_items(released++);
+    if (b.n_lead_items < 0) b.n_lead_items = (int64_t)b.items.size();
     // A projection item may wait for a pair item that another CTA has only
     // just started: allow twice the longest item's time at a conservative 4
     // pairs per CTA per clock (measured: ~4.8 for attraction, ~5.3 directed
@@ -1092,9 +1142,10 @@ int batch_pack(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_g
 }
 
 // Reset the counters and run the first n_items items of the work list with
-// engine tile shape `variant`.
+// engine tile shape `variant`; then, with `project`, the projections if the
+// list holds none (the tuning trials leave K alone).
 int batch_engine(sparkling_ctx *ctx, void *K, int K_dtype, int acc, int variant, int64_t n_items,
-                 cudaStream_t st)
+                 bool project, cudaStream_t st)
 {
     sparkling_ctx::Batch &b = ctx->batch;
     CK(cudaMemsetAsync(at<unsigned int>(ctx, b.o_cnt), 0,
@@ -1121,6 +1172,9 @@ int batch_engine(sparkling_ctx *ctx, void *K, int K_dtype, int acc, int variant,
     e.racc = b.sym || b.one_launch ? at<unsigned long long>(ctx, b.o_racc) : nullptr;
     const int ctas = ctx->sms * engine_ctas_per_sm(acc, K_dtype, variant);
     CK(launch_engine(e, acc, K_dtype, variant, std::min(ctas, b.ctas), st));
+    if (project && b.split_proj)
+        CK(launch_project_batch(e, b.B, b.off[b.B] / b.Ns, b.Ns, momentum_tables(ctx), b.proj_shape,
+                                st));
     return SPARKLING_OK;
 }
 
@@ -1153,7 +1207,7 @@ int batch_device_work(sparkling_ctx *ctx, void *K, int K_dtype, const sparkling_
         CK(cudaMemsetAsync(at<unsigned long long>(ctx, b.o_racc), 0,
                            (size_t)b.off[b.B] * 3 * sizeof(unsigned long long), st));
     }
-    return batch_engine(ctx, K, K_dtype, acc, variant, (int64_t)b.items.size(), st);
+    return batch_engine(ctx, K, K_dtype, acc, variant, (int64_t)b.items.size(), true, st);
 }
 
 // Engine autotuner: time each tile shape on a prefix of the pair items (about
@@ -1175,9 +1229,9 @@ int tune_engine(sparkling_ctx *ctx, void *K, int K_dtype, const sparkling_grid *
     double best_rate = 0.0;
     for (int v = 0; v < kEngineVariants; ++v) {
         if (engine_ctas_per_sm(acc, K_dtype, v) < 1) { cudaGetLastError(); continue; }
-        if ((s = batch_engine(ctx, K, K_dtype, acc, v, n, st))) return s;
+        if ((s = batch_engine(ctx, K, K_dtype, acc, v, n, false, st))) return s;
         CK(cudaEventRecord(e0, st));
-        if ((s = batch_engine(ctx, K, K_dtype, acc, v, n, st))) return s;
+        if ((s = batch_engine(ctx, K, K_dtype, acc, v, n, false, st))) return s;
         CK(cudaEventRecord(e1, st));
         CK(cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -1232,6 +1286,7 @@ SPARKLING_API void sparkling_destroy(sparkling_ctx *ctx)
         cudaFree(ctx->h_rho);
         cudaFree(ctx->d_status);
         cudaFree(ctx->d_small);
+        cudaFree(ctx->d_mom);
         for (auto &p : ctx->pending) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
         for (auto e : ctx->pool) cudaEventDestroy(e);
     }
@@ -1327,7 +1382,7 @@ SPARKLING_API int sparkling_project(sparkling_ctx *ctx, void *K, int K_dtype, in
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Carve cv;
     ProjPlan L;
-    if ((s = plan_project(ctx, K_dtype, Nc, Ns, cv, L))) return s;
+    if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     if ((s = ensure_ws(ctx, cv.off))) return s;
     if ((s = run_project(ctx, K, K_dtype, Nc, Ns, proj, nullptr, 0.0, L, viol_host != nullptr, st)))
         return s;
@@ -1370,7 +1425,7 @@ SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64
     Carve cv;
     if ((s = plan_pairs(ctx, N, grid, acc, false, true, P, cv))) return s;
     ProjPlan L;
-    if ((s = plan_project(ctx, K_dtype, Nc, Ns, cv, L))) return s;
+    if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     if ((s = ensure_ws(ctx, cv.off))) return s;
     // the whole device work of the step, timed as one scope when timing is on
     StepScope whole(ctx, st);
@@ -1426,7 +1481,7 @@ int run_optimize(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t N
     int s;
     if ((s = plan_pairs(ctx, N, grid, acc, false, true, P, cv))) return s;
     ProjPlan L;
-    if ((s = plan_project(ctx, K_dtype, Nc, Ns, cv, L))) return s;
+    if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     const size_t o_kp = cv.take((size_t)n3 * sizeof(double));
     const size_t o_gp = cv.take((size_t)n3 * sizeof(double));
     const size_t o_part = cv.take((size_t)bb_blocks(n3, ctx->sms) * sizeof(double2));
@@ -1606,9 +1661,18 @@ SPARKLING_API int sparkling_step_batched(sparkling_ctx *ctx, int32_t B, const in
     cudaGetLastError();
     if (occ < 1) return fail(ctx, SPARKLING_E_CUDA, "engine kernel cannot be resident");
     const int ctas = ctx->sms * occ;   // the largest wave of any engine shape
+    // FP32 samples: the projections run after the engine in a launch of the
+    // two-float register form, which takes ~1/8 of the FP64 time; as items of
+    // the engine they cost 24 of 248 ms on 16 trajectories (2.4e6 samples),
+    // after it 5.  FP64 samples keep them in the engine, whose pair items
+    // leave the FP64 pipe idle.
+    bool split_proj = K_dtype == SPARKLING_F32;
+    for (int t = 0; t < B && split_proj; ++t)
+        split_proj = project_reg_applies(K_dtype, Ns, proj[t].alpha, proj[t].beta, proj[t].box, 0.0,
+                                         proj[t].pin, proj[t].pin_index, proj[t].n_iter);
     const bool same = b.valid && b.B == B && b.Ns == Ns && b.acc == acc && b.dtype == K_dtype &&
                       b.ctas == ctas && b.items_per_cta == ctx->items_per_cta && b.off == off &&
-                      b.dims == dims && b.one_launch == one_launch;
+                      b.dims == dims && b.one_launch == one_launch && b.split_proj == split_proj;
     if (!same) {
         if (b.exec) { cudaGraphExecDestroy(b.exec); b.exec = nullptr; }
         b = sparkling_ctx::Batch();
@@ -1617,7 +1681,9 @@ SPARKLING_API int sparkling_step_batched(sparkling_ctx *ctx, int32_t B, const in
         b.off = off; b.dims = dims;
         b.one_launch = one_launch;
         b.sym = ctx->rep_symmetric && !one_launch;
-        build_work_list(b, off, grids, ctas, ctx->items_per_cta, b.sym, b.one_launch);
+        b.split_proj = split_proj;
+        b.proj_shape = project_reg_shape(K_dtype, off[B] / Ns, Ns, ctx->sms);
+        build_work_list(b, off, grids, ctas, ctx->items_per_cta, b.sym, b.one_launch, !split_proj);
         b.roles = one_launch;
         if (b.roles) split_work_list(b);
         Carve cv;
@@ -1651,7 +1717,8 @@ SPARKLING_API int sparkling_step_batched(sparkling_ctx *ctx, int32_t B, const in
             b.sym_units = u;
         }
         b.end = cv.off;
-        b.kernels_per_step = 2 + B + (b.sym ? 1 : 0);   // packs, (symmetric repulsion), engine
+        // packs, (symmetric repulsion), engine, (projections)
+        b.kernels_per_step = 2 + B + (b.sym ? 1 : 0) + (b.split_proj ? 1 : 0);
         if ((s = ensure_ws(ctx, b.end))) { b.valid = false; return s; }
         CK(cudaMemcpyAsync(at<EngineItem>(ctx, b.o_items), b.items.data(),
                            b.items.size() * sizeof(EngineItem), cudaMemcpyHostToDevice, st));

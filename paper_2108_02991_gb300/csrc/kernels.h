@@ -239,6 +239,16 @@ cudaError_t launch_bb(const void *K, int dtype, double *Kp, const double *G, dou
                       bool dots, double2 *part, double *out, int sms, cudaStream_t st);
 
 // Projection (project.cu).
+// Momentum factors of the FISTA iterations (1 + mom_it, mom_{it+1}), the same
+// for every row, shot and call: one table a context, as doubles and as
+// two-float sums, kMomentumMax iterations long.
+constexpr int kMomentumMax = 4096;
+struct MomentumTables {
+    const double2 *d;
+    const float4 *f;
+};
+constexpr double kDfHuge = 1.152921504606846976e18;   // 2^60: inputs of the two-float form are cut to it
+
 struct ProjArgs {
     void *K;               // [Nc*Ns][3] in/out
     const double *G;       // optional gradient [Nc*Ns][3]: k = K - eta G
@@ -250,6 +260,7 @@ struct ProjArgs {
     int pin_index, n_iter, check_every;
     double *gstate;        // per-CTA state in global memory (18 * Ns doubles) or null
     int mixed;             // FP32 K, fixed iterations: iterate in FP32 on the displacement
+    MomentumTables mom;
     int *status;
     unsigned long long *viol;  // optional [4] (non-negative doubles as bits)
     int *notconv;          // optional count of shots that did not certify
@@ -259,6 +270,18 @@ bool project_state_in_smem(int Ns);
 int project_block(int Ns);
 int project_ctas_per_sm(int dtype, int Ns);
 cudaError_t launch_project(const ProjArgs &p, int dtype, int grid, cudaStream_t st);
+// The projection with its state in registers (project_reg.cuh): launch shape
+// for Nc shots of Ns samples (samples a thread, CTAs a shot, threads a CTA),
+// or ctas = 0 where it does not apply.
+struct RegShape {
+    int per_thread = 0, ctas = 0, threads = 0;
+};
+bool project_reg_applies(int dtype, int Ns, double alpha, double beta, double box, double tol,
+                         const double *pin, int pin_index, int n_iter);
+RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms);
+// Violations of the result are max-reduced into p.viol when set (a second launch).
+cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, int sms,
+                               cudaStream_t st);
 
 // Persistent engine (engine.cu): one launch runs a work list of pair items
 // (attraction or repulsion of one target tile against a run of grid rows or
@@ -321,6 +344,11 @@ struct EngineArgs {
     float eps2 = kEps2;      // eps^2 (>= kEps2) added to every r^2
     int *status;
 };
+
+// The projections of a batch in one launch of the register form, after the
+// engine has run the pair items (work list without projection items): FP32 K.
+cudaError_t launch_project_batch(const EngineArgs &e, int32_t B, int64_t shots, int Ns,
+                                 const MomentumTables &mom, const RegShape &s, cudaStream_t st);
 
 size_t engine_smem_bytes();
 size_t engine_proj_smem_limit();     // largest 18*Ns*8 that fits the shared-memory union

@@ -1,6 +1,7 @@
 // Per-shot projection onto the gradient-amplitude / slew-rate / box / pin
 // constraint set (paper eq. constraints, Sec. II-D, Suppl. Sec. I) by FISTA on
-// the Fenchel dual of min 1/2 |s - k|^2, in FP64:
+// the Fenchel dual of min 1/2 |s - k|^2, in FP64 (FP32 samples: two-float sums
+// in the register form, project_reg.cuh):
 //   D1 s[n] = s[n+1] - s[n]                 (n < Ns-1)
 //   D2 s[n] = s[n+2] - 2 s[n+1] + s[n]      (n < Ns-2)
 //   s(q)    = pin(clip_box(k - D1^T q1 - D2^T q2))
@@ -10,9 +11,12 @@
 // The output is s(q).  With a gradient G the shot is first stepped:
 // k = K - eta G (eq. proj_grad_descent).
 //
-// FP32 samples may instead (an opt-in of the context) iterate in FP32 on the
-// displacement s - k and the duals (project_shot_mixed); FP64 is the default
-// for every sample type.
+// Fixed iterations run in the register form (project_reg.cuh) up to 8192
+// samples a shot.  What follows is the form with its state in memory, for
+// converged mode, longer shots, more iterations than the momentum table holds
+// and radii outside the two-float range; there FP32 samples may (an opt-in of
+// the context) iterate in FP32 on the displacement s - k and the duals
+// (project_shot_mixed), else in FP64.
 //
 // One CTA per shot (grid-stride over shots).  The 18 per-sample FP64 arrays
 // (k, s, y1, y2, q1, q2; x, y, z each, structure of arrays so that a warp
@@ -20,11 +24,14 @@
 // per-CTA global scratch region otherwise; the code is the same through
 // generic pointers.  Each iteration is two phases separated by barriers:
 // S computes s from the duals, Z updates the duals from s.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <cmath>
 #include <cstdint>
 
 #include "kernels.h"
 #include "project_dev.cuh"
+#include "project_reg.cuh"
 #include "ptx.cuh"
 
 namespace sparkling {
@@ -69,7 +76,244 @@ __global__ void __launch_bounds__(kProjMaxThreads) project_kernel(const ProjArgs
     }
 }
 
+// Threads a CTA of the register form may have: M = 1 takes 80 registers a
+// thread, M = 2 takes 128.
+constexpr __host__ __device__ int reg_max_threads(int M) { return M == 1 ? 768 : 512; }
+constexpr int kRegMaxCtas = 8;                 // portable cluster size
+
+// The slots and neighbours of the calling warp; zeroed, and every CTA of the
+// cluster running, on return.
+template <class R, int M, bool CL> struct RegEdges {
+    EdgeSlot<R> *mine, *to_right = nullptr, *to_left = nullptr;
+    bool first, last;
+    int C, rank;
+
+    __device__ RegEdges(EdgeSlot<R> *slots)
+    {
+        namespace cg = cooperative_groups;
+        const cg::cluster_group cl = cg::this_cluster();
+        C = CL ? (int)cl.num_blocks() : 1;
+        rank = CL ? (int)cl.block_rank() : 0;
+        const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+        first = rank == 0 && warp == 0;
+        last = rank == C - 1 && warp == warps - 1;
+        mine = &slots[warp];
+        if (warp < warps - 1) to_right = &slots[warp + 1];
+        else if (CL && !last) to_right = cl.map_shared_rank(&slots[0], rank + 1);
+        if (warp > 0) to_left = &slots[warp - 1];
+        else if (CL && !first) to_left = cl.map_shared_rank(&slots[warps - 1], rank - 1);
+        for (int q = threadIdx.x; q < warps * kSlotWords; q += blockDim.x)
+            reinterpret_cast<double *>(slots)[q] = 0.0;
+        sync();
+    }
+    __device__ __forceinline__ static void sync()
+    {
+        if (CL) cooperative_groups::this_cluster().sync();
+        else if (blockDim.x == 32) __syncwarp();
+        else __syncthreads();
+    }
+    __device__ int first_sample() const { return (rank * (int)blockDim.x + (int)threadIdx.x) * M; }
+
+    template <class LoadK, class Store>
+    __device__ __forceinline__ void project(const RegShot &sh, const MomentumTables &mom,
+                                            LoadK loadk, Store store)
+    {
+        project_registers<R, M>(sh, mom, first_sample(), mine, to_right, to_left, first, last,
+                                [] { sync(); }, loadk, store);
+        sync();                // the slots are free again (and no CTA leaves early)
+    }
+};
+
+// One shot per cluster (CL) or CTA, grid-stride over shots; thread t of CTA
+// rank r owns samples (r * blockDim + t) * M + [0, M).
+template <class R, int M, typename KT, bool CL>
+__global__ void __launch_bounds__(reg_max_threads(M)) project_reg_kernel(const ProjArgs p)
+{
+    __shared__ EdgeSlot<R> slots[reg_max_threads(M) / 32];
+    RegEdges<R, M, CL> edges(slots);
+    RegShot sh;
+    sh.Ns = p.Ns; sh.n_iter = p.n_iter; sh.pin_index = p.pin_index;
+    sh.alpha = p.alpha; sh.beta = p.beta; sh.box = p.box;
+    for (int c = 0; c < 3; ++c) sh.pin[c] = p.pin[c];
+    KT *K = static_cast<KT *>(p.K);
+    const double *G = p.G;
+    const double eta = p.eta;
+    for (int64_t shot = blockIdx.x / edges.C; shot < p.Nc; shot += gridDim.x / edges.C) {
+        const int64_t off = shot * (int64_t)p.Ns;
+        edges.project(sh, p.mom,
+            [&](int m, double *kv) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    kv[c] = (double)K[3 * (off + m) + c];
+                    if (G) kv[c] -= eta * G[3 * (off + m) + c];
+                }
+            },
+            [&](int m, const R *s) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) K[3 * (off + m) + c] = (KT)r_value(s[c]);
+            });
+    }
+}
+
+// The shots of a batch's trajectories (FP32 samples), after the engine: the
+// gradient is formed from the trajectory's slots and repulsion totals in the
+// order of the engine's projection items.  A trajectory whose pair items did
+// not all finish (a bounded wait ran out) is left as it is.
+template <int M, bool CL>
+__global__ void __launch_bounds__(reg_max_threads(M)) project_batch_kernel(const EngineArgs e,
+                                                                           int B, int64_t shots,
+                                                                           int Ns,
+                                                                           MomentumTables mom)
+{
+    __shared__ EdgeSlot<Df> slots[reg_max_threads(M) / 32];
+    RegEdges<Df, M, CL> edges(slots);
+    for (int64_t shot = blockIdx.x / edges.C; shot < shots; shot += gridDim.x / edges.C) {
+        int lo = 0, hi = B - 1;                   // the largest t with off_t <= shot * Ns
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (e.traj[mid].off <= shot * Ns) lo = mid;
+            else hi = mid - 1;
+        }
+        const EngineTraj &tr = e.traj[lo];
+        if (e.done[lo] < (unsigned int)tr.n_pair_items) continue;   // the whole cluster alike
+        RegShot sh;
+        sh.Ns = Ns; sh.n_iter = tr.n_iter; sh.pin_index = tr.pin_index;
+        sh.alpha = tr.alpha; sh.beta = tr.beta; sh.box = tr.box;
+        for (int c = 0; c < 3; ++c) sh.pin[c] = tr.pin[c];
+        float *K = static_cast<float *>(e.K) + 3 * shot * (int64_t)Ns;
+        const int64_t first = shot * Ns - tr.off;               // local sample index
+        const dacc4 *part = e.part + tr.part_off;
+        const double invN = 1.0 / (double)tr.N, eta = tr.eta;
+        const int slots_n = tr.slots, ach = tr.a_chunks;
+        edges.project(sh, mom,
+            [&](int m, double *kv) {
+                const int64_t i = first + m, tile = i / kTile, l = i - tile * kTile;
+                const dacc4 *p = part + tile * slots_n * kTile + l;
+                double g[3] = {0.0, 0.0, 0.0}, r[3] = {0.0, 0.0, 0.0};
+                for (int s = 0; s < slots_n; ++s) {
+                    const dacc4 v = p[(int64_t)s * kTile];
+                    if (s < ach) { g[0] += v.x; g[1] += v.y; g[2] += v.z; }
+                    else { r[0] += v.x; r[1] += v.y; r[2] += v.z; }
+                }
+                if (e.racc) {
+                    const unsigned long long *q = e.racc + 3 * (tr.off + i);
+                    for (int c = 0; c < 3; ++c) r[c] = (double)(long long)q[c] / kFixScale;
+                }
+                for (int c = 0; c < 3; ++c) kv[c] = (double)K[3 * m + c] - eta * (g[c] - r[c] * invN);
+            },
+            [&](int m, const Df *s) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) K[3 * m + c] = r_value(s[c]);
+            });
+    }
+}
+
+template <typename KT>
+__global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
+{
+    ShotParams sp;
+    sp.Ns = p.Ns;
+    sp.alpha = p.alpha; sp.beta = p.beta; sp.box = p.box; sp.tol = 0.0; sp.margin = 0.0;
+    for (int c = 0; c < 3; ++c) sp.pin[c] = p.pin[c];
+    sp.pin_index = p.pin_index; sp.n_iter = p.n_iter; sp.check_every = 0;
+    sp.viol = p.viol; sp.notconv = nullptr;
+    for (int64_t shot = blockIdx.x; shot < p.Nc; shot += gridDim.x)
+        record_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * (int64_t)p.Ns, sp);
+}
+
+template <bool CL> void *reg_fn(int dtype, int M)
+{
+    if (dtype == 0)
+        return M == 1 ? reinterpret_cast<void *>(project_reg_kernel<Df, 1, float, CL>)
+                      : reinterpret_cast<void *>(project_reg_kernel<Df, 2, float, CL>);
+    return M == 1 ? reinterpret_cast<void *>(project_reg_kernel<double, 1, double, CL>)
+                  : reinterpret_cast<void *>(project_reg_kernel<double, 2, double, CL>);
+}
+
 } // namespace
+
+bool project_reg_applies(int dtype, int Ns, double alpha, double beta, double box, double tol,
+                         const double *pin, int pin_index, int n_iter)
+{
+    if (tol > 0.0 || n_iter > kMomentumMax || Ns > kRegMaxCtas * 2 * reg_max_threads(2)) return false;
+    if (dtype != 0) return true;
+    // two-float form: radii and box whose squares and low parts stay normal
+    constexpr double lo = 1.0 / (1ll << 40), hi = (double)(1ll << 40);
+    auto radius_ok = [&](double r) { return std::isinf(r) || (r >= lo && r <= hi); };
+    if (!radius_ok(alpha) || !radius_ok(beta) || !(box >= lo && box <= hi)) return false;
+    for (int c = 0; c < 3; ++c)
+        if (pin_index >= 0 && !(std::fabs(pin[c]) <= hi)) return false;
+    return true;
+}
+
+// Shape rule.  Two floats (FP32 samples): issue-bound, so M = 2 (the fewest
+// instructions a sample), and CTAs of at most 256 threads -- two on an SM
+// cover each other's barriers: 4096 shots of 2560 samples take 24.5 ms as 5
+// CTAs of 256 threads, 30.1 ms as 3 of 448.  Shots of up to 128 samples are
+// bound by the latency of one warp's chain: M = 1 (32 x 64: 86 against 107 us).
+// FP64: bound by the FP64 pipe, which every warp of an SM shares.  M = 1 costs
+// ~10 % more operations but pads less and has the shorter chain; it is taken
+// where the shots do not fill the GPU (37 x 129: 379 against 531 us; 300 x
+// 700: 2.80 against 2.53 ms).  One CTA up to 1024 samples (a cluster barrier
+// costs ~0.4 us: 300 x 700 as 2 CTAs takes 2.79 ms), else at most 256 threads.
+RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms)
+{
+    RegShape s;
+    const bool fp64 = dtype != 0;
+    s.per_thread = fp64 ? (Nc <= sms && Ns <= 256 ? 1 : 2) : (Ns <= 128 ? 1 : 2);
+    const int one = fp64 ? 1024 : 512;            // samples a single CTA takes
+    s.ctas = Ns <= one ? 1 : (Ns + 511) / 512;
+    if (s.ctas > kRegMaxCtas) s.ctas = kRegMaxCtas;
+    const int per = s.ctas * s.per_thread;
+    s.threads = ((Ns + per - 1) / per + 31) / 32 * 32;
+    return s;
+}
+
+namespace {
+
+cudaError_t launch_reg(void *fn, const RegShape &s, int64_t shots, void **args, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    const int64_t most = ((int64_t)1 << 20) / s.ctas;
+    cfg.gridDim = dim3((unsigned)((shots < most ? shots : most) * s.ctas));
+    cfg.blockDim = dim3((unsigned)s.threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)s.ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = s.ctas > 1 ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+} // namespace
+
+cudaError_t launch_project_batch(const EngineArgs &e, int32_t B, int64_t shots, int Ns,
+                                 const MomentumTables &mom, const RegShape &s, cudaStream_t st)
+{
+    void *fn = s.ctas > 1 ? (s.per_thread == 1 ? reinterpret_cast<void *>(project_batch_kernel<1, true>)
+                                               : reinterpret_cast<void *>(project_batch_kernel<2, true>))
+                          : (s.per_thread == 1 ? reinterpret_cast<void *>(project_batch_kernel<1, false>)
+                                               : reinterpret_cast<void *>(project_batch_kernel<2, false>));
+    int b = B;
+    MomentumTables m = mom;
+    void *args[] = {const_cast<EngineArgs *>(&e), &b, &shots, &Ns, &m};
+    return launch_reg(fn, s, shots, args, st);
+}
+
+cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, int sms,
+                               cudaStream_t st)
+{
+    void *fn = s.ctas > 1 ? reg_fn<true>(dtype, s.per_thread) : reg_fn<false>(dtype, s.per_thread);
+    void *args[] = {const_cast<ProjArgs *>(&p)};
+    cudaError_t e = launch_reg(fn, s, p.Nc, args, st);
+    if (e != cudaSuccess || !p.viol) return e;
+    const unsigned g = (unsigned)(p.Nc < sms * 8 ? p.Nc : sms * 8);
+    if (dtype == 0) violation_kernel<float><<<g, 256, 0, st>>>(p);
+    else violation_kernel<double><<<g, 256, 0, st>>>(p);
+    return cudaGetLastError();
+}
 
 size_t project_state_bytes(int Ns) { return (size_t)18 * Ns * sizeof(double); }
 

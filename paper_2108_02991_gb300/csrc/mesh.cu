@@ -4,9 +4,9 @@
 //
 // The kernel splits exactly: d/r = d/r erfc(r/sigma) + d/r erf(r/sigma),
 // r = |d|_eps.  The short-range part decays like a Gaussian and is summed
-// directly over the pairs closer than rc, found through a cell list (cells
-// of side >= rc/2, samples sorted by cell).  The long-range part is smooth and
-// is summed on a mesh:
+// directly over the pairs closer than rc, found through the bounding boxes of
+// clusters of samples sorted along a Hilbert curve.  The long-range part is smooth and is
+// summed on a mesh:
 //   1. every sample spreads a unit charge to 4 x 4 x 4 nodes with cubic
 //      B-spline weights (64-bit fixed-point atomics: exact, order-free);
 //   2. the charge mesh (M^3 nodes, zero-padded to L = 2M per axis) is
@@ -25,7 +25,6 @@
 #include <cuda_runtime.h>
 #include <cufft.h>
 #include <cub/device/device_radix_sort.cuh>
-#include <cub/device/device_scan.cuh>
 
 #include <algorithm>
 #include <cmath>
@@ -188,7 +187,8 @@ __device__ __forceinline__ NodeWeights node_weights(float4 p, double x0, double 
     return nw;
 }
 
-// Unit charges of the samples on the M^3 charge mesh (fixed point).
+// Unit charges of the samples (in curve order) on the M^3 charge mesh (fixed
+// point: the order of the additions does not matter).
 __global__ void spread_kernel(const float4 *__restrict__ pos, int64_t N, unsigned long long *Q,
                               double x0, double inv_h, int M, int *status)
 {
@@ -244,10 +244,12 @@ __global__ void spectrum_product_kernel(cufftComplex *out, const cufftComplex *_
 // Long-range sums gathered from the convolved fields (L^3 boxes; node n of
 // the mesh is box index n) -- the force x, y, z fields, or the potential
 // field alone for the energy -- plus the short-range fixed-point sums
-// ([N][3] or [N][1]): out = S + L.
+// ([3][N] or [1][N]): out = S + L.
+// Thread k takes the k-th sample of the curve order (neighbours read the same
+// nodes) and writes it at its own index idx[k].
 template <bool ENERGY>
-__global__ void gather_kernel(const float4 *__restrict__ pos, int64_t N,
-                              const float *__restrict__ phi, int64_t box, int L, double x0,
+__global__ void gather_kernel(const float4 *__restrict__ pos, const int *__restrict__ idx,
+                              int64_t N, const float *__restrict__ phi, int64_t box, int L, double x0,
                               double inv_h, int M, const unsigned long long *__restrict__ shortr,
                               dacc4 *out)
 {
@@ -278,276 +280,430 @@ __global__ void gather_kernel(const float4 *__restrict__ pos, int64_t N,
             r.x = r.y = r.z = 0.0;
             r.w = (double)(long long)shortr[i] * (1.0 / kFix) + (double)acc[0];
         } else {
-            r.x = (double)(long long)shortr[3 * i] * (1.0 / kFix) + (double)acc[0];
-            r.y = (double)(long long)shortr[3 * i + 1] * (1.0 / kFix) + (double)acc[NC > 1 ? 1 : 0];
-            r.z = (double)(long long)shortr[3 * i + 2] * (1.0 / kFix) + (double)acc[NC > 2 ? 2 : 0];
+            r.x = (double)(long long)shortr[i] * (1.0 / kFix) + (double)acc[0];
+            r.y = (double)(long long)shortr[N + i] * (1.0 / kFix) + (double)acc[NC > 1 ? 1 : 0];
+            r.z = (double)(long long)shortr[2 * N + i] * (1.0 / kFix) + (double)acc[NC > 2 ? 2 : 0];
             r.w = 0.0;
         }
-        out[i] = r;
+        out[idx[i]] = r;
     }
 }
 
 // ---- short-range part ------------------------------------------------------
+//
+// The samples are sorted along a Hilbert curve (10 bits an axis; a Morton curve
+// jumps, and the boxes of samples on both sides of a jump are large).  A
+// cluster is 32 consecutive samples; clusters, runs of 32 clusters and runs of 32 of those
+// keep their bounding boxes (levels 0, 1, 2).  Where samples crowd -- the
+// centre, which every shot crosses -- their clusters are small, so the boxes
+// follow the density by themselves.
+//
+// A warp holds a group of two clusters, one target of each a lane, and finds
+// the clusters behind it in the order with a box within rc of the group's, 32
+// tests at a time through the levels.  Two near clusters at a time, a source
+// of each a lane, meet the group: the sources and their sums rotate one lane a
+// step, so every unordered pair is evaluated once and counts for both samples
+// (the pair term is odd).  The two sources of a lane share 64-bit registers
+// (paired FP32).  Inside the group every ordered pair is evaluated.  A cluster
+// near one half of the group only meets that half.
+//
+// Bound: the FP32 and SFU pipes together (22 lane operations and three SFU
+// results an unordered pair; at four targets a lane ncu has them 67 and 61 %
+// busy, the warps of an SM moving through the same step in phase).  Measured
+// against the cell list before it (directed pairs, cells of rc/3, every source
+// of 49 neighbour rows tested against 64 targets): 1e7 samples, 256 cells
+// 176 -> 71 ms; 1e6 samples on spokes, 128 cells 250 -> 80 ms.  On the way, 1e7 /
+// 1e6 samples: directed with the sources culled against the boxes 124 / 152 ms,
+// symmetric pairs 133 / 90, Hilbert instead of Morton order 82 / 77 ms; with four
+// targets a lane 85 ms (larger boxes, half the shuffles).
 
-__device__ __forceinline__ int cell_coord(float x, float x0, float inv_cs, int nc)
+constexpr int kCluster = 32;
+
+// Spread the low 10 bits of v to every third bit.
+__device__ __forceinline__ unsigned int spread3(unsigned int v)
 {
-    int c = (int)floorf((x - x0) * inv_cs);
-    return c < 0 ? 0 : (c >= nc ? nc - 1 : c);
+    v &= 0x3ffu;
+    v = (v | (v << 16)) & 0x030000ffu;
+    v = (v | (v << 8)) & 0x0300f00fu;
+    v = (v | (v << 4)) & 0x030c30c3u;
+    v = (v | (v << 2)) & 0x09249249u;
+    return v;
 }
 
-__global__ void cell_keys_kernel(const float4 *__restrict__ pos, int64_t N, float x0, float inv_cs,
-                                 int nc, unsigned int *keys, int *vals)
+__device__ __forceinline__ unsigned int grid_coord(float x, float x0, float inv)
+{
+    const int c = (int)floorf((x - x0) * inv);
+    return (unsigned int)(c < 0 ? 0 : (c > 1023 ? 1023 : c));
+}
+
+// Index of a cell on the Hilbert curve of the 1024^3 grid, by the exchange and
+// inversion of axes bit by bit (Skilling, "Programming the Hilbert curve", 2004).
+__device__ __forceinline__ unsigned int hilbert_key(unsigned int x, unsigned int y, unsigned int z)
+{
+    unsigned int a[3] = {x, y, z};
+#pragma unroll
+    for (int bit = 9; bit > 0; --bit) {
+        const unsigned int low = (1u << bit) - 1u;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const unsigned int set = 0u - ((a[c] >> bit) & 1u);       // all ones where the bit is set
+            const unsigned int swap = (a[0] ^ a[c]) & low & ~set;     // exchange with axis 0, or
+            a[0] ^= swap | (low & set);                               // invert axis 0
+            a[c] ^= swap;
+        }
+    }
+    a[1] ^= a[0];                                                     // Gray code
+    a[2] ^= a[1];
+    unsigned int flip = 0u;
+#pragma unroll
+    for (int bit = 9; bit > 0; --bit) flip ^= (0u - ((a[2] >> bit) & 1u)) & ((1u << bit) - 1u);
+    return spread3(a[0] ^ flip) << 2 | spread3(a[1] ^ flip) << 1 | spread3(a[2] ^ flip);
+}
+
+__global__ void curve_keys_kernel(const float4 *__restrict__ pos, int64_t N, float x0, float inv,
+                                  unsigned int *keys, int *vals)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float4 p = pos[i];
-        const int cx = cell_coord(p.x, x0, inv_cs, nc), cy = cell_coord(p.y, x0, inv_cs, nc),
-                  cz = cell_coord(p.z, x0, inv_cs, nc);
-        keys[i] = (unsigned int)((cz * nc + cy) * nc + cx);
+        keys[i] = hilbert_key(grid_coord(p.x, x0, inv), grid_coord(p.y, x0, inv),
+                              grid_coord(p.z, x0, inv));
         vals[i] = (int)i;
     }
 }
 
-// Cell ranges [start, end) of the sorted keys (cells without samples keep
-// start = end = 0) and the samples' positions in sorted order.
-__global__ void cell_ranges_kernel(const unsigned int *__restrict__ keys,
-                                   const int *__restrict__ idx, const float4 *__restrict__ pos,
-                                   int64_t N, int *start, int *end, float4 *spos)
+struct Box {
+    float4 lo, hi;
+};
+
+__device__ __forceinline__ Box empty_box()
 {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned int c = keys[k];
-        if (k == 0 || keys[k - 1] != c) start[c] = (int)k;
-        if (k == N - 1 || keys[k + 1] != c) end[c] = (int)(k + 1);
-        spos[k] = pos[idx[k]];
+    const float inf = __int_as_float(0x7f800000);
+    return {make_float4(inf, inf, inf, 0.f), make_float4(-inf, -inf, -inf, 0.f)};
+}
+
+// Union of the boxes of the lanes of each aligned group of W lanes.
+template <int W> __device__ __forceinline__ void box_union(Box &b)
+{
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) {
+        b.lo.x = fminf(b.lo.x, __shfl_xor_sync(0xffffffffu, b.lo.x, o));
+        b.lo.y = fminf(b.lo.y, __shfl_xor_sync(0xffffffffu, b.lo.y, o));
+        b.lo.z = fminf(b.lo.z, __shfl_xor_sync(0xffffffffu, b.lo.z, o));
+        b.hi.x = fmaxf(b.hi.x, __shfl_xor_sync(0xffffffffu, b.hi.x, o));
+        b.hi.y = fmaxf(b.hi.y, __shfl_xor_sync(0xffffffffu, b.hi.y, o));
+        b.hi.z = fmaxf(b.hi.z, __shfl_xor_sync(0xffffffffu, b.hi.z, o));
     }
 }
 
-// erfc(x), x >= 0: Abramowitz & Stegun 7.1.26 polynomial in t = 1/(1 + p x)
-// times exp(-x^2) (returned separately, the energy needs it too).
-__device__ __forceinline__ float erfc_as(float x, float &gauss)
+// The samples' positions in sorted order and the boxes of their clusters (one
+// warp a cluster).  Coordinates are multiplied by `unit`, a power of two (no
+// rounding), which puts sigma into [1/2, 1).
+__global__ void sorted_clusters_kernel(const int *__restrict__ idx, const float4 *__restrict__ pos,
+                                       int64_t N, int64_t n0, float unit, float4 *spos, Box *boxes)
 {
-    const float t = __frcp_rn(fmaf(0.3275911f, x, 1.f));
-    float poly = fmaf(t, 1.061405429f, -1.453152027f);
-    poly = fmaf(t, poly, 1.421413741f);
-    poly = fmaf(t, poly, -0.284496736f);
-    poly = fmaf(t, poly, 0.254829592f);
-    gauss = __expf(-x * x);
-    return t * poly * gauss;
-}
-
-// Cells have side >= rc / kCellReach, so the pairs closer than rc lie in the
-// (2 kCellReach + 1)^3 cells around a sample's cell (smaller cells: fewer
-// candidate pairs beyond rc).
-constexpr int kCellReach = 3;
-constexpr int kRowSpan = 2 * kCellReach + 1;
-constexpr int kRows = kRowSpan * kRowSpan;
-
-// Sorted range [j0, j1) of the sources in row r (0 .. kRows-1: dz, dy in
-// -kCellReach .. kCellReach) of the cells around cell (cx, cy, cz): the
-// x-neighbours of a row are consecutive cells, so their samples are one
-// contiguous range.
-__device__ __forceinline__ bool row_range(int cx, int cy, int cz, int r, int nc,
-                                          const int *__restrict__ start,
-                                          const int *__restrict__ end, int &j0, int &j1)
-{
-    const int z = cz + r / kRowSpan - kCellReach, y = cy + r % kRowSpan - kCellReach;
-    if (z < 0 || z >= nc || y < 0 || y >= nc) return false;
-    const int xa = cx >= kCellReach ? cx - kCellReach : 0;
-    const int xb = cx < nc - kCellReach ? cx + kCellReach : nc - 1;
-    const int base = (z * nc + y) * nc;
-    j0 = -1;
-    for (int x = xa; x <= xb; ++x) {
-        const int s = start[base + x], e = end[base + x];
-        if (s < e) {
-            if (j0 < 0) j0 = s;
-            j1 = e;
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; c < n0; c += warps) {
+        const int64_t k = c * kCluster + lane;
+        Box b = empty_box();
+        if (k < N) {
+            float4 p = pos[idx[k]];
+            p.x *= unit; p.y *= unit; p.z *= unit;
+            spos[k] = p;
+            b.lo = b.hi = p;
         }
+        box_union<32>(b);
+        if (lane == 0) boxes[c] = b;
     }
-    return j0 >= 0;
+}
+
+// Boxes of the runs of 32 boxes of the level below (n of them).
+__global__ void parent_boxes_kernel(const Box *__restrict__ below, int64_t n, Box *boxes)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t up = (n + 31) / 32, warps = (int64_t)gridDim.x * blockDim.x / 32;
+    for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; c < up; c += warps) {
+        const int64_t k = c * 32 + lane;
+        Box b = k < n ? below[k] : empty_box();
+        box_union<32>(b);
+        if (lane == 0) boxes[c] = b;
+    }
+}
+
+struct ShortArgs {
+    const float4 *spos;
+    const Box *boxes;            // levels 0, 1, 2 one after the other
+    int64_t N, n0, n1, n2;
+    int64_t groups;              // ceil(N / kGroup)
+    int parts;                   // parts of the sources of one group (a power of two)
+    unsigned long long *queue;
+    float rc2, rc2_cull;         // cut-off, compared with d^2 + eps2; the same for boxes, rounded up
+    float eps2;                  // eps^2, at least kEps2
+    float p;                     // 0.3275911 / sigma
+    float gauss;                 // -log2(e) / sigma^2
+    float nspi;                  // -sigma / sqrt(pi)
+    float to_fix;                // sums to fixed point: 2^32 (and the energy back to its unit)
+    unsigned long long *acc;     // [NV][N] fixed-point sums, curve order
+};
+
+__device__ __forceinline__ float gap(float lo, float hi, float tlo, float thi)
+{
+    return fmaxf(fmaxf(lo - thi, tlo - hi), 0.f);
+}
+
+// Whether box b may hold a point within rc of the box t (never false where
+// one does: rc2_cull is rc^2 rounded up by more than the test's rounding).
+__device__ __forceinline__ bool box_near(const Box &b, const Box &t, float rc2_cull)
+{
+    const float gx = gap(b.lo.x, b.hi.x, t.lo.x, t.hi.x), gy = gap(b.lo.y, b.hi.y, t.lo.y, t.hi.y),
+                gz = gap(b.lo.z, b.hi.z, t.lo.z, t.hi.z);
+    return fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= rc2_cull;
 }
 
 constexpr int kShortThreads = 128;               // 4 warps, each takes its own items
-constexpr int kShortChunk = 64;                  // targets per item (2 per lane of a warp)
-constexpr int kShortSlice = 4096;                // sources per item at most
+constexpr int kT = 2;                            // targets a lane
+constexpr int kGroup = 32 * kT;
+constexpr int kFoldSteps = 64;                   // cluster pairs summed in FP32 (4096 sources a target)
 
-// Items of cell c: ceil(n_c / kShortChunk) target chunks times the source
-// slices of its kRows rows.
-__global__ void count_items_kernel(const int *__restrict__ start, const int *__restrict__ end,
-                                   int nc, int *counts, int *slices)
+struct ShortTargets {
+    f2 x[kT], y[kT], z[kT];                      // each target in both halves
+    f2 ax[kT], ay[kT], az[kT];                   // its sums over the two sources' halves
+};
+
+__device__ __forceinline__ void add_fix(unsigned long long *p, float v, float to_fix)
 {
-    const int ncell = nc * nc * nc;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-        const int n = end[c] - start[c];
-        int cnt = 0, sl = 0;
-        if (n > 0) {
-            const int cx = c % nc, cy = (c / nc) % nc, cz = c / (nc * nc);
-            for (int r = 0; r < kRows; ++r) {
-                int j0, j1;
-                if (row_range(cx, cy, cz, r, nc, start, end, j0, j1))
-                    sl += (j1 - j0 + kShortSlice - 1) / kShortSlice;
+    const long long x = __float2ll_rn(v * to_fix);
+    if (x) atomicAdd(p, (unsigned long long)x);
+}
+
+// The group's targets against two clusters of sources (q0, q1: the lane's).
+// erfc(x) is a polynomial in t = 1/(1 + p x) times exp(-x^2): 22 FP32 lane
+// operations and three SFU results a pair, which load the two pipes alike (a
+// polynomial for log2 erfc needs two SFU results and 24 operations: 7 % slower).
+// SYM: the sources' sums are added to their totals as well.
+// Pairs of samples with |d| < rc only; the self pair adds nothing to the force
+// and g_short(0) to the energy.
+// T0, TN: the targets that take part (both halves of the group, or one).
+template <bool ENERGY, bool SYM, int T0, int TN>
+__device__ __forceinline__ void short_step(const ShortArgs &a, ShortTargets &T, float4 q0, float4 q1,
+                                           int64_t k0, int64_t k1, bool ok0, bool ok1)
+{
+    const int lane = threadIdx.x & 31, from = (lane + 1) & 31;
+    f2 SX = f2_pack(q0.x, q1.x), SY = f2_pack(q0.y, q1.y), SZ = f2_pack(q0.z, q1.z);
+    f2 BX = f2_pack(0.f, 0.f), BY = BX, BZ = BX;
+    // paired constants, kept in registers (as constant-bank operands of the
+    // paired instructions they cost 10 %)
+    auto both = [](float v) { return f2_pack(v, v); };
+    const f2 E2 = both(a.eps2);
+    const f2 ONE = both(1.f), P = both(a.p), GA = both(a.gauss), NSPI = both(a.nspi);
+    const f2 C5 = both(1.061405429f), C4 = both(-1.453152027f), C3 = both(1.421413741f),
+             C2 = both(-0.284496736f), C1 = both(0.254829592f);
+    for (int step = 0; step < 32; ++step) {
+#pragma unroll
+        for (int t = T0; t < T0 + TN; ++t) {
+            const f2 DX = f2_sub(T.x[t], SX), DY = f2_sub(T.y[t], SY), DZ = f2_sub(T.z[t], SZ);
+            const f2 R2 = f2_fma(DX, DX, f2_fma(DY, DY, f2_fma(DZ, DZ, E2)));
+            float r2a, r2b, ea, eb;
+            f2_unpack(R2, r2a, r2b);
+            const f2 RI = f2_pack(rsqrt_sfu(r2a), rsqrt_sfu(r2b));
+            const f2 R = f2_mul(R2, RI);
+            float da, db;
+            f2_unpack(f2_fma(R, P, ONE), da, db);
+            const f2 TT = f2_pack(rcp_sfu(da), rcp_sfu(db));
+            f2_unpack(f2_mul(R2, GA), ea, eb);
+            ea = r2a < a.rc2 ? ex2_sfu(ea) : 0.f;
+            eb = r2b < a.rc2 ? ex2_sfu(eb) : 0.f;
+            const f2 G = f2_pack(ea, eb);
+            const f2 EC = f2_mul(f2_mul(TT, G), f2_fma(TT, f2_fma(TT, f2_fma(TT, f2_fma(TT, C5, C4),
+                                                                          C3), C2), C1));
+            if (ENERGY) {
+                const f2 E = f2_fma(R, EC, f2_mul(NSPI, G));
+                T.ax[t] = f2_add(T.ax[t], E);
+                if (SYM) BX = f2_add(BX, E);
+            } else {
+                const f2 W = f2_mul(EC, RI);
+                T.ax[t] = f2_fma(DX, W, T.ax[t]);
+                T.ay[t] = f2_fma(DY, W, T.ay[t]);
+                T.az[t] = f2_fma(DZ, W, T.az[t]);
+                if (SYM) {
+                    BX = f2_fma(DX, W, BX);
+                    BY = f2_fma(DY, W, BY);
+                    BZ = f2_fma(DZ, W, BZ);
+                }
             }
-            cnt = ((n + kShortChunk - 1) / kShortChunk) * sl;
         }
-        counts[c] = cnt;
-        slices[c] = sl;
-    }
-}
-
-// The short-range work list, numbered on the device: cell c owns items
-// [offsets[c], offsets[c] + counts[c]) (an exclusive scan of the counts),
-// ceil(n_c / kShortChunk) target chunks times slices[c] source slices of
-// its neighbour rows.  The kernels read its length on the device: the items
-// below the stored list's capacity are written by fill_items_kernel (one
-// thread per item) and read by the short-range kernel, which decodes any
-// item beyond the capacity itself.
-// Item u -> (targets t0, tn; sources s0, sn), all sorted positions.
-__device__ int4 item_at(int64_t u, const int *__restrict__ offsets, const int *__restrict__ slices,
-                        const int *__restrict__ start, const int *__restrict__ end, int nc)
-{
-    const int ncell = nc * nc * nc;
-    int lo = 0, hi = ncell - 1;                // largest c with offsets[c] <= u
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((int64_t)offsets[mid] <= u) lo = mid;
-        else hi = mid - 1;
-    }
-    const int c = lo;
-    const int local = (int)(u - offsets[c]), sl = slices[c];
-    int4 it = make_int4(0, 0, 0, 0);
-    if (sl <= 0 || local < 0) return it;
-    const int k = local / sl;
-    int rs = local % sl;
-    const int cx = c % nc, cy = (c / nc) % nc, cz = c / (nc * nc);
-    it.x = start[c] + k * kShortChunk;
-    it.y = min(kShortChunk, end[c] - it.x);
-    for (int r = 0; r < kRows; ++r) {
-        int j0, j1;
-        if (!row_range(cx, cy, cz, r, nc, start, end, j0, j1)) continue;
-        const int ns = (j1 - j0 + kShortSlice - 1) / kShortSlice;
-        if (rs < ns) {
-            it.z = j0 + rs * kShortSlice;
-            it.w = min(kShortSlice, j1 - it.z);
-            break;
+        // the sources and their sums move one lane down
+        SX = __shfl_sync(0xffffffffu, SX, from);
+        SY = __shfl_sync(0xffffffffu, SY, from);
+        SZ = __shfl_sync(0xffffffffu, SZ, from);
+        if (SYM) {
+            BX = __shfl_sync(0xffffffffu, BX, from);
+            if (!ENERGY) {
+                BY = __shfl_sync(0xffffffffu, BY, from);
+                BZ = __shfl_sync(0xffffffffu, BZ, from);
+            }
         }
-        rs -= ns;
     }
-    return it;
+    if (SYM) {                                   // back home after 32 steps; the force term is odd
+        float u, v;
+        f2_unpack(BX, u, v);
+        if (ok0) add_fix(a.acc + k0, ENERGY ? u : -u, a.to_fix);
+        if (ok1) add_fix(a.acc + k1, ENERGY ? v : -v, a.to_fix);
+        if (!ENERGY) {
+            f2_unpack(BY, u, v);
+            if (ok0) add_fix(a.acc + a.N + k0, -u, a.to_fix);
+            if (ok1) add_fix(a.acc + a.N + k1, -v, a.to_fix);
+            f2_unpack(BZ, u, v);
+            if (ok0) add_fix(a.acc + 2 * a.N + k0, -u, a.to_fix);
+            if (ok1) add_fix(a.acc + 2 * a.N + k1, -v, a.to_fix);
+        }
+    }
 }
 
-// The list's length, and its first `cap` items stored (grid-stride).
-__global__ void fill_items_kernel(const int *__restrict__ counts, const int *__restrict__ offsets,
-                                  const int *__restrict__ slices, const int *__restrict__ start,
-                                  const int *__restrict__ end, int nc, int64_t cap, int4 *items,
-                                  long long *total_out)
+// A lane of `todo` whose cluster is near the halves `want`, or any.
+__device__ __forceinline__ int pick(unsigned int todo, int near, int want)
 {
-    const int ncell = nc * nc * nc;
-    const int64_t total = (int64_t)offsets[ncell - 1] + counts[ncell - 1];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *total_out = total;
-    const int64_t n = total < cap ? total : cap;
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
-         u += (int64_t)gridDim.x * blockDim.x)
-        items[u] = item_at(u, offsets, slices, start, end, nc);
+    const unsigned int same = __ballot_sync(0xffffffffu, near == want) & todo;
+    return __ffs(same ? same : todo) - 1;
 }
 
-// Short-range pair term of target p and source q, added to f (force) or
-// f[0] (energy): pairs with |d| < rc only; the self pair adds nothing to the
-// force and g_short(0) to the energy.
+// Persistent warps take items (group, part) from a queue; part p of P takes
+// every P-th near level-1 run, so that no item is long where samples crowd.
+// FP32 sums go to 64-bit fixed-point totals (exact, order-free).
 template <bool ENERGY>
-__device__ __forceinline__ void short_pair(const float4 p, const float4 q, float rc2,
-                                           float inv_sigma, float spi, float eps2, float *f)
-{
-    const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    if (d2 < rc2) {
-        const float re2 = d2 + eps2;
-        const float ri = rsqrt_sfu(fmaxf(re2, kEps2));
-        const float r = re2 * ri;
-        float gauss;
-        const float ec = erfc_as(r * inv_sigma, gauss);
-        if (ENERGY) {
-            f[0] += fmaf(r, ec, -spi * gauss);
-        } else {
-            const float w = ec * ri;
-            f[0] = fmaf(dx, w, f[0]);
-            f[1] = fmaf(dy, w, f[1]);
-            f[2] = fmaf(dz, w, f[2]);
-        }
-    }
-}
-
-// One item: targets [it.x, it.x + it.y) (two per lane) against sources
-// [it.z, it.z + it.w) of the sorted positions, the sums added to the targets'
-// fixed-point accumulators.
-template <bool ENERGY>
-__device__ __forceinline__ void short_item(const int4 it, int lane, const float4 *__restrict__ spos,
-                                           const int *__restrict__ idx, float rc2, float inv_sigma,
-                                           float spi, float eps2, unsigned long long *acc)
+__global__ void __launch_bounds__(kShortThreads, 5) short_items_kernel(const ShortArgs a)
 {
     constexpr int NV = ENERGY ? 1 : 3;
-    float4 p[2];
-    bool ok[2];
-    float f[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-    for (int t = 0; t < 2; ++t) {
-        const int l = lane + 32 * t;
-        ok[t] = l < it.y;
-        p[t] = ok[t] ? spos[it.x + l] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const float4 *src = spos + it.z;
-#pragma unroll 4
-    for (int j = 0; j < it.w; ++j) {
-        const float4 q = __ldg(src + j);
-        short_pair<ENERGY>(p[0], q, rc2, inv_sigma, spi, eps2, f[0]);
-        short_pair<ENERGY>(p[1], q, rc2, inv_sigma, spi, eps2, f[1]);
-    }
-    for (int t = 0; t < 2; ++t) {
-        if (!ok[t]) continue;
-        unsigned long long *a = acc + (int64_t)idx[it.x + lane + 32 * t] * NV;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const long long x = __float2ll_rn(f[t][v] * 4294967296.0f);
-            if (x) atomicAdd(a + v, (unsigned long long)x);
-        }
-    }
-}
-
-// Persistent warps take items from a queue: kShortChunk targets of one cell
-// (two per lane) against up to kShortSlice sources of one neighbour row.
-// The lanes of a warp read the same source at the same time (one broadcast
-// load serves 64 pairs); the item sums are added to the targets' 64-bit
-// fixed-point accumulators (exact, order-free).  Small items keep the lanes
-// busy where cells hold few samples.  The length of the list is read on the
-// device; items below `cap` come from the stored list, the rest are decoded
-// here: nothing about the work list goes through the host, so an evaluation
-// can be captured in a CUDA graph.
-template <bool ENERGY>
-__global__ void __launch_bounds__(kShortThreads) short_items_kernel(
-    const int4 *__restrict__ items, int64_t cap, const int *__restrict__ counts,
-    const int *__restrict__ offsets, const int *__restrict__ slices, const int *__restrict__ start,
-    const int *__restrict__ end, int nc, unsigned int *queue, const float4 *__restrict__ spos,
-    const int *__restrict__ idx, float rc2, float inv_sigma, float spi, float eps2,
-    unsigned long long *acc)
-{
+    constexpr unsigned int kAll = 0xffffffffu;
+    __shared__ Box halves[kShortThreads / 32][2];
     const int lane = threadIdx.x & 31;
-    const int ncell = nc * nc * nc;
-    const int64_t total = (int64_t)offsets[ncell - 1] + counts[ncell - 1];
+    const Box *box0 = a.boxes, *box1 = box0 + a.n0, *box2 = box1 + a.n1;
+    const unsigned long long total = (unsigned long long)a.groups * a.parts;
+    // samples that do not exist: beyond every cut-off of the others
+    const float4 no_target = make_float4(1e18f, 1e18f, 1e18f, 0.f);
+    const float4 no_source = make_float4(-1e18f, -1e18f, -1e18f, 0.f);
     for (;;) {
-        int64_t u = 0;
-        if (lane == 0) u = atomicAdd(queue, 1u);
-        u = __shfl_sync(0xffffffffu, u, 0);
+        unsigned long long u = 0;
+        if (lane == 0) u = atomicAdd(a.queue, 1ull);
+        u = __shfl_sync(kAll, u, 0);
         if (u >= total) break;
-        int4 it;
-        if (u < cap) {
-            it = items[u];
-        } else {                               // beyond the stored list: decode it here
-            if (lane == 0) it = item_at(u, offsets, slices, start, end, nc);
-            it.x = __shfl_sync(0xffffffffu, it.x, 0);
-            it.y = __shfl_sync(0xffffffffu, it.y, 0);
-            it.z = __shfl_sync(0xffffffffu, it.z, 0);
-            it.w = __shfl_sync(0xffffffffu, it.w, 0);
+        const int part = (int)(u / a.groups);
+        const int64_t g = (int64_t)(u % a.groups), first = g * kGroup;
+        ShortTargets T;
+        Box half[2] = {empty_box(), empty_box()};
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+            Box &tb = half[t / (kT / 2)];
+            const int64_t k = first + t * 32 + lane;
+            const bool ok = k < a.N;
+            const float4 p = ok ? a.spos[k] : no_target;
+            T.x[t] = f2_pack(p.x, p.x);
+            T.y[t] = f2_pack(p.y, p.y);
+            T.z[t] = f2_pack(p.z, p.z);
+            T.ax[t] = T.ay[t] = T.az[t] = f2_pack(0.f, 0.f);
+            if (ok) {
+                tb.lo = make_float4(fminf(tb.lo.x, p.x), fminf(tb.lo.y, p.y), fminf(tb.lo.z, p.z), 0.f);
+                tb.hi = make_float4(fmaxf(tb.hi.x, p.x), fmaxf(tb.hi.y, p.y), fmaxf(tb.hi.z, p.z), 0.f);
+            }
         }
-        if (it.y > 0 && it.w > 0)
-            short_item<ENERGY>(it, lane, spos, idx, rc2, inv_sigma, spi, eps2, acc);
+        box_union<32>(half[0]);
+        box_union<32>(half[1]);
+        // the halves' boxes wait in shared memory; the group's stays at hand
+        __syncwarp();
+        if (lane == 0) {
+            halves[threadIdx.x >> 5][0] = half[0];
+            halves[threadIdx.x >> 5][1] = half[1];
+        }
+        __syncwarp();
+        const Box *hb = halves[threadIdx.x >> 5];
+        Box tb;
+        tb.lo = make_float4(fminf(half[0].lo.x, half[1].lo.x), fminf(half[0].lo.y, half[1].lo.y),
+                            fminf(half[0].lo.z, half[1].lo.z), 0.f);
+        tb.hi = make_float4(fmaxf(half[0].hi.x, half[1].hi.x), fmaxf(half[0].hi.y, half[1].hi.y),
+                            fmaxf(half[0].hi.z, half[1].hi.z), 0.f);
+        int steps = 0;
+        auto fold = [&]() {
+#pragma unroll
+            for (int t = 0; t < kT; ++t) {
+                const int64_t k = first + t * 32 + lane;
+                float u0, v0;
+                f2_unpack(T.ax[t], u0, v0);
+                if (k < a.N) add_fix(a.acc + k, u0 + v0, a.to_fix);
+                if (NV > 1) {
+                    f2_unpack(T.ay[t], u0, v0);
+                    if (k < a.N) add_fix(a.acc + a.N + k, u0 + v0, a.to_fix);
+                    f2_unpack(T.az[t], u0, v0);
+                    if (k < a.N) add_fix(a.acc + 2 * a.N + k, u0 + v0, a.to_fix);
+                }
+                T.ax[t] = T.ay[t] = T.az[t] = f2_pack(0.f, 0.f);
+            }
+            steps = 0;
+        };
+        // the group's own pairs, directed (part 0)
+        if (part == 0) {
+            for (int h = 0; h < kT; h += 2) {
+                const int64_t k0 = first + h * 32 + lane, k1 = k0 + 32;
+                short_step<ENERGY, false, 0, kT>(a, T, k0 < a.N ? a.spos[k0] : no_source,
+                                                 k1 < a.N ? a.spos[k1] : no_source, 0, 0, false,
+                                                 false);
+                ++steps;
+            }
+        }
+        // the clusters behind the group, two at a time
+        const int64_t behind = (g + 1) * kT;       // first cluster behind
+        int64_t held = -1;                         // a near cluster waiting for a second one,
+        int held_near = 0;                         // and the halves it is near to (bits)
+        auto meet = [&](int64_t c0, int64_t c1, int near) {
+            const int64_t k0 = c0 * kCluster + lane, k1 = c1 * kCluster + lane;
+            const bool ok0 = k0 < a.N, ok1 = c1 >= 0 && k1 < a.N;
+            const float4 q0 = ok0 ? a.spos[k0] : no_source, q1 = ok1 ? a.spos[k1] : no_source;
+            if (near == 3)
+                short_step<ENERGY, true, 0, kT>(a, T, q0, q1, k0, k1, ok0, ok1);
+            else if (near == 1)
+                short_step<ENERGY, true, 0, kT / 2>(a, T, q0, q1, k0, k1, ok0, ok1);
+            else
+                short_step<ENERGY, true, kT / 2, kT / 2>(a, T, q0, q1, k0, k1, ok0, ok1);
+            if (++steps == kFoldSteps) fold();
+        };
+        int ordinal = 0;
+        for (int64_t b2 = behind / 1024 / 32 * 32; b2 < a.n2; b2 += 32) {
+            unsigned int m2 = __ballot_sync(kAll, b2 + lane < a.n2 && (b2 + lane + 1) * 1024 > behind &&
+                                                      box_near(box2[b2 + lane], tb, a.rc2_cull));
+            while (m2) {
+                const int64_t b1 = (b2 + __ffs(m2) - 1) * 32;
+                m2 &= m2 - 1;
+                unsigned int m1 = __ballot_sync(kAll, b1 + lane < a.n1 && (b1 + lane + 1) * 32 > behind &&
+                                                          box_near(box1[b1 + lane], tb, a.rc2_cull));
+                while (m1) {
+                    const int64_t b0 = (b1 + __ffs(m1) - 1) * 32;
+                    m1 &= m1 - 1;
+                    if ((ordinal++ & (a.parts - 1)) != part) continue;
+                    int near = 0;
+                    if (b0 + lane < a.n0 && b0 + lane >= behind) {
+                        const Box b = box0[b0 + lane];
+                        near = (box_near(b, hb[0], a.rc2_cull) ? 1 : 0) |
+                               (box_near(b, hb[1], a.rc2_cull) ? 2 : 0);
+                    }
+                    // clusters near the same halves meet them together
+                    unsigned int todo = __ballot_sync(kAll, near != 0);
+                    while (todo) {
+                        const int l = held < 0 ? __ffs(todo) - 1 : pick(todo, near, held_near);
+                        todo &= ~(1u << l);
+                        const int ln = __shfl_sync(kAll, near, l);
+                        if (held < 0) {
+                            held = b0 + l;
+                            held_near = ln;
+                        } else {
+                            meet(held, b0 + l, held_near | ln);
+                            held = -1;
+                        }
+                    }
+                }
+            }
+        }
+        if (held >= 0) meet(held, -1, held_near);
+        if (steps > 0) fold();
     }
 }
 
@@ -580,7 +736,7 @@ template <typename T> cudaError_t grow(T *&p, size_t &cap, size_t bytes)
 struct MeshState {
     MeshConfig cfg;          // the mesh the spectra were built for
     bool built = false;
-    int M = 0, L = 0, nc = 0;
+    int M = 0, L = 0;
     double x0 = 0.0;
     cufftComplex *spectra = nullptr;   // 4 kernel spectra on the L box (scaled by 1/L^3)
     size_t spectra_cap = 0;
@@ -591,16 +747,13 @@ struct MeshState {
     float *box = nullptr; size_t box_cap = 0;           // charges, then 4 fields
     cufftComplex *qhat = nullptr; size_t qhat_cap = 0;
     cufftComplex *tmp = nullptr; size_t tmp_cap = 0;
-    unsigned int *keys = nullptr; size_t keys_cap = 0;   // 2N keys, 2N values
-    int *vals = nullptr; size_t vals_cap = 0;
-    int *ranges = nullptr; size_t ranges_cap = 0;        // start[nc^3], end[nc^3]
-    float4 *spos = nullptr; size_t spos_cap = 0;
-    unsigned long long *shortr = nullptr; size_t shortr_cap = 0;   // fixed point [N][3]
-    int *cellwork = nullptr; size_t cellwork_cap = 0;   // counts, slices, offsets [ncell] each
-    int4 *items = nullptr; size_t items_cap = 0;        // the stored part of the work list
-    int64_t items_n = -1;                               // the sample count it was sized for
-    unsigned long long *dsmall = nullptr;               // [0]: item queue, [1]: list length
-    int short_ctas[2] = {0, 0};                         // persistent CTAs (gradient, energy)
+    unsigned int *keys = nullptr; size_t keys_cap = 0;   // 2N keys
+    int *vals = nullptr; size_t vals_cap = 0;            // 2N indices
+    float4 *spos = nullptr; size_t spos_cap = 0;         // samples in curve order
+    Box *boxes = nullptr; size_t boxes_cap = 0;          // levels 0, 1, 2
+    unsigned long long *shortr = nullptr; size_t shortr_cap = 0;   // fixed point [3][N], curve order
+    unsigned long long *queue = nullptr;                 // item queue
+    int short_ctas[2] = {0, 0};                          // persistent CTAs (gradient, energy)
     void *cub = nullptr; size_t cub_cap = 0;
 };
 
@@ -611,9 +764,8 @@ void mesh_state_destroy(MeshState *m)
     if (!m) return;
     if (m->plans) { cufftDestroy(m->r2c); cufftDestroy(m->c2r); }
     cudaFree(m->spectra); cudaFree(m->Q); cudaFree(m->box); cudaFree(m->qhat); cudaFree(m->tmp);
-    cudaFree(m->keys); cudaFree(m->vals); cudaFree(m->ranges); cudaFree(m->spos);
-    cudaFree(m->shortr); cudaFree(m->cub); cudaFree(m->cellwork); cudaFree(m->items);
-    cudaFree(m->dsmall);
+    cudaFree(m->keys); cudaFree(m->vals); cudaFree(m->spos); cudaFree(m->boxes);
+    cudaFree(m->shortr); cudaFree(m->cub); cudaFree(m->queue);
     delete m;
 }
 
@@ -762,10 +914,6 @@ cudaError_t mesh_build(MeshState *m, const MeshConfig &c, int sms, cudaStream_t 
     m->M = M;
     m->L = L;
     m->x0 = c.lo - g * h;
-    const double span = M * h;
-    m->nc = (int)std::floor(span * kCellReach / c.rc);
-    if (m->nc < 1) m->nc = 1;
-    if (m->nc > 512) m->nc = 512;
     m->built = true;
     *what = "";
     return done(cudaSuccess);
@@ -774,8 +922,7 @@ cudaError_t mesh_build(MeshState *m, const MeshConfig &c, int sms, cudaStream_t 
 // Repulsion sums of the N packed samples into out[i] = (sum d/r, sum |d|_eps)
 // over all j (directed, the self pair included as eps in the potential).
 // Asynchronous: once the buffers have their size for N (the first call of a
-// sample count allocates them and waits once for the length of its
-// short-range work list), a call only enqueues work on `st` and can be
+// sample count allocates them), a call only enqueues work on `st` and can be
 // captured.
 // no_alloc (a call under stream capture): return cudaErrorStreamCaptureUnsupported
 // instead of growing a buffer.
@@ -784,32 +931,27 @@ cudaError_t mesh_eval(MeshState *m, const float4 *pos, int64_t N, bool energy, d
                       bool no_alloc)
 {
     const MeshConfig &c = m->cfg;
-    const int M = m->M, L = m->L, nc = m->nc;
+    const int M = m->M, L = m->L;
     const int64_t nm = (int64_t)M * M * M, nl = (int64_t)L * L * L, nlc = (int64_t)L * L * (L / 2 + 1);
     const int nfield = energy ? 1 : 3;
     const int NV = energy ? 1 : 3;
-    const int ncell = nc * nc * nc;
+    const int64_t n0 = (N + kCluster - 1) / kCluster, n1 = (n0 + 31) / 32, n2 = (n1 + 31) / 32;
     const double h = (c.hi - c.lo) / c.n_cells;
     cudaError_t err;
     *what = "mesh evaluation buffers";
-    size_t sort_bytes = 0, scan_bytes = 0;
-    int end_bit = 1;
-    while (((int64_t)1 << end_bit) < ncell) ++end_bit;
+    size_t sort_bytes = 0;
+    constexpr int kKeyBits = 30;
     cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, m->keys, m->keys, m->vals, m->vals,
-                                    (int)N, 0, end_bit, st);
-    cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, m->cellwork, m->cellwork, ncell, st);
-    const size_t cub_bytes = std::max(sort_bytes, scan_bytes);
+                                    (int)N, 0, kKeyBits, st);
     if (no_alloc &&
         (nm * sizeof(unsigned long long) > m->Q_cap ||
          (size_t)(nfield + 1) * nl * sizeof(float) > m->box_cap ||
          nlc * sizeof(cufftComplex) > m->qhat_cap || nlc * sizeof(cufftComplex) > m->tmp_cap ||
          (size_t)2 * N * sizeof(unsigned int) > m->keys_cap ||
-         (size_t)2 * N * sizeof(int) > m->vals_cap ||
-         (size_t)2 * ncell * sizeof(int) > m->ranges_cap ||
-         (size_t)N * sizeof(float4) > m->spos_cap ||
+         (size_t)2 * N * sizeof(int) > m->vals_cap || (size_t)N * sizeof(float4) > m->spos_cap ||
+         (size_t)(n0 + n1 + n2) * sizeof(Box) > m->boxes_cap ||
          (size_t)N * 3 * sizeof(unsigned long long) > m->shortr_cap ||
-         (size_t)3 * ncell * sizeof(int) > m->cellwork_cap || cub_bytes + 256 > m->cub_cap ||
-         !m->dsmall || !m->short_ctas[0] || m->items_n != N))
+         sort_bytes + 256 > m->cub_cap || !m->queue || !m->short_ctas[0]))
         return cudaErrorStreamCaptureUnsupported;
 
     if ((err = grow(m->Q, m->Q_cap, nm * sizeof(unsigned long long))) ||
@@ -818,13 +960,12 @@ cudaError_t mesh_eval(MeshState *m, const float4 *pos, int64_t N, bool energy, d
         (err = grow(m->tmp, m->tmp_cap, nlc * sizeof(cufftComplex))) ||
         (err = grow(m->keys, m->keys_cap, (size_t)2 * N * sizeof(unsigned int))) ||
         (err = grow(m->vals, m->vals_cap, (size_t)2 * N * sizeof(int))) ||
-        (err = grow(m->ranges, m->ranges_cap, (size_t)2 * ncell * sizeof(int))) ||
         (err = grow(m->spos, m->spos_cap, (size_t)N * sizeof(float4))) ||
+        (err = grow(m->boxes, m->boxes_cap, (size_t)(n0 + n1 + n2) * sizeof(Box))) ||
         (err = grow(m->shortr, m->shortr_cap, (size_t)N * 3 * sizeof(unsigned long long))) ||
-        (err = grow(m->cellwork, m->cellwork_cap, (size_t)3 * ncell * sizeof(int))) ||
-        (err = grow(m->cub, m->cub_cap, cub_bytes + 256)))
+        (err = grow(m->cub, m->cub_cap, sort_bytes + 256)))
         return err;
-    if (!m->dsmall && (err = cudaMalloc(&m->dsmall, 2 * sizeof(unsigned long long)))) return err;
+    if (!m->queue && (err = cudaMalloc(&m->queue, sizeof(unsigned long long)))) return err;
     if (!m->short_ctas[0]) {
         int a = 0, b = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, short_items_kernel<false>, kShortThreads, 0);
@@ -835,69 +976,53 @@ cudaError_t mesh_eval(MeshState *m, const float4 *pos, int64_t N, bool energy, d
     if (cufftSetStream(m->r2c, st) != CUFFT_SUCCESS || cufftSetStream(m->c2r, st) != CUFFT_SUCCESS)
         return cudaErrorUnknown;
     *what = "mesh evaluation";
-    const int gN = grid_for(N, sms), gC = grid_for(ncell, sms);
+    const int gN = grid_for(N, sms);
     int nk = 0;
-    // short-range part: samples sorted by cell, work items, pair sums
-    const float cs = (float)(M * h / nc);
-    cell_keys_kernel<<<gN, kMeshThreads, 0, st>>>(pos, N, (float)m->x0, 1.f / cs, nc, m->keys,
-                                                  m->vals);
+    // short-range part: samples sorted, boxes, pair sums
+    curve_keys_kernel<<<gN, kMeshThreads, 0, st>>>(pos, N, (float)m->x0, (float)(1024.0 / (M * h)),
+                                                    m->keys, m->vals);
     if ((err = cub::DeviceRadixSort::SortPairs(m->cub, sort_bytes, m->keys, m->keys + N, m->vals,
-                                               m->vals + N, (int)N, 0, end_bit, st)))
+                                               m->vals + N, (int)N, 0, kKeyBits, st)))
         return err;
-    if ((err = cudaMemsetAsync(m->ranges, 0, (size_t)2 * ncell * sizeof(int), st))) return err;
-    int *start = m->ranges, *end = m->ranges + ncell;
-    cell_ranges_kernel<<<gN, kMeshThreads, 0, st>>>(m->keys + N, m->vals + N, pos, N, start, end,
-                                                    m->spos);
-    int *counts = m->cellwork, *slices = counts + ncell, *offsets = slices + ncell;
-    count_items_kernel<<<gC, kMeshThreads, 0, st>>>(start, end, nc, counts, slices);
-    if ((err = cub::DeviceScan::ExclusiveSum(m->cub, scan_bytes, counts, offsets, ncell, st)))
+    const int *idx = m->vals + N;
+    Box *box1 = m->boxes + n0, *box2 = box1 + n1;
+    int exponent = 0;
+    std::frexp(c.sigma, &exponent);                // sigma = f 2^exponent, f in [1/2, 1)
+    const double unit = std::ldexp(1.0, -exponent), sigma = c.sigma * unit, eps = c.eps * unit;
+    sorted_clusters_kernel<<<grid_for(n0 * 32, sms), kMeshThreads, 0, st>>>(
+        idx, pos, N, n0, (float)unit, m->spos, m->boxes);
+    parent_boxes_kernel<<<grid_for(n1 * 32, sms), kMeshThreads, 0, st>>>(m->boxes, n0, box1);
+    parent_boxes_kernel<<<grid_for(n2 * 32, sms), kMeshThreads, 0, st>>>(box1, n1, box2);
+    ShortArgs a{};
+    a.spos = m->spos; a.boxes = m->boxes;
+    a.N = N; a.n0 = n0; a.n1 = n1; a.n2 = n2;
+    a.groups = (N + kGroup - 1) / kGroup;
+    a.parts = 1;
+    while (a.parts < 32 && a.groups * a.parts < ((int64_t)1 << 20)) a.parts *= 2;
+    a.queue = m->queue;
+    const double rc = c.rc * unit;
+    a.eps2 = std::max((float)(eps * eps), kEps2);
+    a.rc2 = (float)(rc * rc + eps * eps);
+    a.rc2_cull = (float)(rc * rc * (1.0 + 1e-5));
+    a.p = (float)(0.3275911 / sigma);
+    a.gauss = (float)(-1.4426950408889634 / (sigma * sigma));
+    a.nspi = (float)(-sigma * 0.56418958354775628);
+    a.to_fix = (float)(4294967296.0 / (energy ? unit : 1.0));
+    a.acc = m->shortr;
+    if ((err = cudaMemsetAsync(m->queue, 0, sizeof(unsigned long long), st)) ||
+        (err = cudaMemsetAsync(m->shortr, 0, (size_t)N * NV * sizeof(unsigned long long), st)))
         return err;
-    unsigned int *queue = reinterpret_cast<unsigned int *>(m->dsmall);
-    long long *d_total = reinterpret_cast<long long *>(m->dsmall + 1);
-    if (!no_alloc && m->items_n != N) {
-        // The first evaluation of a sample count sizes the stored list: it
-        // waits once for the list's length and keeps room for half as many
-        // again (the list changes as the samples move; any items beyond the
-        // room are decoded by the short-range kernel).  The list is not
-        // reallocated while the sample count stays the same.
-        fill_items_kernel<<<1, 32, 0, st>>>(counts, offsets, slices, start, end, nc, 0, nullptr,
-                                            d_total);
-        ++nk;
-        long long total = 0;
-        if ((err = cudaMemcpyAsync(&total, d_total, sizeof(long long), cudaMemcpyDeviceToHost, st)) ||
-            (err = cudaStreamSynchronize(st)))
-            return err;
-        const size_t want = (size_t)std::max<long long>(total, 0);
-        const size_t bytes = (want + want / 2 + 1024) * sizeof(int4);
-        cudaFree(m->items);
-        m->items = nullptr;
-        m->items_cap = 0;
-        m->items_n = -1;
-        if ((err = cudaMalloc(&m->items, bytes))) return err;
-        m->items_cap = bytes;
-        m->items_n = N;
-    }
-    const int64_t cap = (int64_t)(m->items_cap / sizeof(int4));
-    if ((err = cudaMemsetAsync(queue, 0, sizeof(unsigned int), st))) return err;
-    fill_items_kernel<<<grid_for(std::max<int64_t>(cap, 1), sms), kMeshThreads, 0, st>>>(
-        counts, offsets, slices, start, end, nc, cap, m->items, d_total);
-    if ((err = cudaMemsetAsync(m->shortr, 0, (size_t)N * NV * sizeof(unsigned long long), st)))
-        return err;
-    const float rc2 = (float)(c.rc * c.rc), inv_sigma = (float)(1.0 / c.sigma);
-    const float spi = (float)(c.sigma * 0.56418958354775628);
-    const float eps2 = (float)(c.eps * c.eps);
+    const int64_t warps_needed = a.groups * a.parts;
+    const int ctas = (int)std::min<int64_t>(m->short_ctas[energy ? 1 : 0], (warps_needed + 3) / 4);
     if (energy)
-        short_items_kernel<true><<<m->short_ctas[1], kShortThreads, 0, st>>>(
-            m->items, cap, counts, offsets, slices, start, end, nc, queue, m->spos, m->vals + N,
-            rc2, inv_sigma, spi, eps2, m->shortr);
+        short_items_kernel<true><<<ctas, kShortThreads, 0, st>>>(a);
     else
-        short_items_kernel<false><<<m->short_ctas[0], kShortThreads, 0, st>>>(
-            m->items, cap, counts, offsets, slices, start, end, nc, queue, m->spos, m->vals + N,
-            rc2, inv_sigma, spi, eps2, m->shortr);
+        short_items_kernel<false><<<ctas, kShortThreads, 0, st>>>(a);
     nk += 6;
     // long-range part
     if ((err = cudaMemsetAsync(m->Q, 0, nm * sizeof(unsigned long long), st))) return err;
-    spread_kernel<<<gN, kMeshThreads, 0, st>>>(pos, N, m->Q, m->x0, 1.0 / h, M, status);
+    spread_kernel<<<gN, kMeshThreads, 0, st>>>(m->spos, N, m->Q, m->x0 * unit, 1.0 / (h * unit), M,
+                                               status);
     charges_to_box_kernel<<<grid_for(nl, sms), kMeshThreads, 0, st>>>(m->Q, m->box, M, L);
     if (cufftExecR2C(m->r2c, m->box, m->qhat) != CUFFT_SUCCESS) return cudaErrorUnknown;
     for (int k = 0; k < nfield; ++k) {
@@ -908,11 +1033,13 @@ cudaError_t mesh_eval(MeshState *m, const float4 *pos, int64_t N, bool energy, d
             return cudaErrorUnknown;
     }
     if (energy)
-        gather_kernel<true><<<gN, kMeshThreads, 0, st>>>(pos, N, m->box + nl, nl, L, m->x0,
-                                                         1.0 / h, M, m->shortr, out);
+        gather_kernel<true><<<gN, kMeshThreads, 0, st>>>(m->spos, idx, N, m->box + nl, nl, L,
+                                                         m->x0 * unit, 1.0 / (h * unit), M,
+                                                         m->shortr, out);
     else
-        gather_kernel<false><<<gN, kMeshThreads, 0, st>>>(pos, N, m->box + nl, nl, L, m->x0,
-                                                          1.0 / h, M, m->shortr, out);
+        gather_kernel<false><<<gN, kMeshThreads, 0, st>>>(m->spos, idx, N, m->box + nl, nl, L,
+                                                          m->x0 * unit, 1.0 / (h * unit), M,
+                                                          m->shortr, out);
     nk += 3 + nfield + 1;
     *launches = nk;
     *what = "";

@@ -105,6 +105,21 @@ __device__ __forceinline__ float rsqrt_sfu(float x)
     return y;
 }
 
+// MUFU.RCP and MUFU.EX2: approximate 1/x and 2^x, flushing subnormals.
+__device__ __forceinline__ float rcp_sfu(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float ex2_sfu(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Paired FP32 arithmetic (two lanes of a 64-bit register, one instruction:
 // the f32x2 forms of add, sub, mul and fma of sm_100 and later).
 typedef unsigned long long f2;

@@ -18,7 +18,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsparkling.so")
-SOURCES = ["api.cu", "pairs.cu", "repulsion.cu", "repulsion_sym.cu", "project.cu", "noalloc.cu",
+SOURCES = ["api.cu", "pairs.cu", "repulsion.cu", "repulsion_sym.cu", "repulsion_small.cu", "project.cu", "noalloc.cu",
            "engine.cu", "field.cu", "driver.cu", "mesh.cu"]
 HEADERS = ["kernels.h", "ptx.cuh", "pair_dev.cuh", "project_dev.cuh", "project_reg.cuh", "sym_dev.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -27,6 +27,10 @@ using namespace sparkling;
 // persistent engine (measured faster on the 1e7-sample workload).
 constexpr int64_t kStepEngineMin = (int64_t)1 << 22;
 
+// Up to this many samples the repulsion runs directed over the whole GPU
+// (repulsion_small.cu) instead of on pairs of 1024-sample tiles.
+constexpr int64_t kSmallRepulsion = 20480;
+
 struct sparkling_ctx {
     int device = 0;
     bool inited = false;
@@ -66,6 +70,7 @@ struct sparkling_ctx {
     bool rep_symmetric = true;     // repulsion: symmetric kernel (else the directed shapes)
     int occ_sym[2][kSymVariants] = {};
     int sym_choice = -1;           // shape of the symmetric kernel (tuned or pinned; -1: none)
+    bool pin_sym = false;          // sym_choice was pinned by sparkling_set_shape
     int pin_attr = -1;             // attraction shape pinned by sparkling_set_shape
     std::string tune_log;
     // batched step: cached work list, workspace layout and CUDA graph
@@ -702,12 +707,19 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
         int s = build_field(ctx, g, st);
         if (s) return s;
     }
+    const bool mesh_mode = ctx->rep_mode == SPARKLING_REPULSION_MESH;
+    // few samples: the directed kernel over the whole GPU, unless a shape of
+    // the symmetric one was pinned
+    const bool small = !mesh_mode && P.N <= kSmallRepulsion && !ctx->pin_sym;
+    // fixed-point totals of the repulsion, cleared by the pack
+    const bool totals = small || (!mesh_mode && ctx->rep_symmetric);
+    const int64_t n_totals = totals ? P.N * (energy ? 1 : 3) : 0;
     {
         LaunchScope ls(ctx, SPARKLING_KERNEL_PACK, st);
-        CK(launch_pack_positions(K, K_dtype, P.N, pos, ctx->d_status, ctx->sms, st));
-        CK(launch_pack_grid(g->rho, P.nx, P.ny, P.nz, P.gxp, g->lo, g->hi, rho, coords,
-                            ctx->d_status, ctx->sms, st));
-        ls.done(2);
+        CK(launch_pack(K, K_dtype, P.N, pos, g->rho, P.nx, P.ny, P.nz, P.gxp, g->lo, g->hi, rho,
+                       coords, at<unsigned long long>(ctx, P.o_racc), n_totals, ctx->d_status,
+                       ctx->sms, st));
+        ls.done();
     }
     AttrArgs aa{};
     aa.tgt = pos; aa.N = P.N; aa.rho = rho; aa.coords = coords;
@@ -721,10 +733,9 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     ra.pos = pos; ra.N = P.N; ra.part = at<dacc4>(ctx, P.o_partr);
     ra.status = ctx->d_status;
     ra.eps2 = aa.eps2;
-    const bool mesh_mode = ctx->rep_mode == SPARKLING_REPULSION_MESH;
     const bool need_a = !field_mode && attr_choice_of(ctx, acc, P.gxp) < 0,
-               need_r = !mesh_mode && !ctx->rep_symmetric && ctx->rep_choice[rep_acc(acc)] < 0,
-               need_s = !mesh_mode && ctx->rep_symmetric && ctx->sym_choice < 0;
+               need_r = !mesh_mode && !small && !ctx->rep_symmetric && ctx->rep_choice[rep_acc(acc)] < 0,
+               need_s = !mesh_mode && !small && ctx->rep_symmetric && ctx->sym_choice < 0;
     if (ctx->autotune && (need_a || need_r || need_s)) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         CK(cudaStreamIsCapturing(st, &cap));
@@ -734,6 +745,9 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
             if (s) return s;
             const int va = attr_choice_of(ctx, acc, P.gxp), vr = ctx->rep_choice[rep_acc(acc)];
             set_splits(ctx, P, acc, energy, va < 0 ? kAttrDefault : va, vr < 0 ? kRepDefault : vr);
+            if (need_s)      // the trials added into the totals
+                CK(cudaMemsetAsync(at<unsigned long long>(ctx, P.o_racc), 0,
+                                   (size_t)n_totals * sizeof(unsigned long long), st));
         }
     }
     aa.sp = P.spa;
@@ -771,6 +785,11 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, what);
         ls.done(nk);
+    } else if (small) {
+        racc = at<unsigned long long>(ctx, P.o_racc);
+        LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
+        CK(launch_repulsion_small(pos, P.N, ra.eps2, energy, racc, ctx->sms, st));
+        ls.done();
     } else if (ctx->rep_symmetric) {
         // every unordered pair once, exact fixed-point totals
         racc = at<unsigned long long>(ctx, P.o_racc);
@@ -780,7 +799,6 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
         sa.ctas = (int64_t)ctx->sms * ctx->occ_sym[energy ? 1 : 0][sv];
         sa.acc = racc; sa.status = ctx->d_status; sa.eps2 = ra.eps2;
         LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
-        CK(cudaMemsetAsync(racc, 0, (size_t)P.N * (energy ? 1 : 3) * sizeof(unsigned long long), st));
         CK(launch_repulsion_sym(sa, energy, sv, st));
         ls.done();
     } else {
@@ -1903,6 +1921,7 @@ SPARKLING_API int sparkling_set_autotune(sparkling_ctx *ctx, int enable)
         ctx->rep_choice[0] = ctx->rep_choice[1] = -1;
         for (auto &row : ctx->engine_choice) row[0] = row[1] = -1;
         ctx->sym_choice = -1;
+        ctx->pin_sym = false;
         ctx->pin_attr = -1;
         ctx->tune_log.clear();
         ctx->autotune = true;
@@ -1925,6 +1944,7 @@ SPARKLING_API int sparkling_set_shape(sparkling_ctx *ctx, int kernel, int varian
             return fail(ctx, SPARKLING_E_INVAL, "repulsion shape %d not in -1..%d", variant,
                         kSymVariants - 1);
         ctx->sym_choice = variant;
+        ctx->pin_sym = variant >= 0;
         return SPARKLING_OK;
     }
     return fail(ctx, SPARKLING_E_INVAL, "kernel %d has no selectable shape", kernel);

@@ -182,6 +182,11 @@ cudaError_t launch_pack_positions(const void *K, int dtype, int64_t N, float4 *o
 cudaError_t launch_pack_grid(const float *rho, int nx, int ny, int nz, int gxp, double lo,
                              double hi, float *rho_out, float *coords, int *status, int sms,
                              cudaStream_t st);
+// Both in one launch, and n_zero words of `zero` cleared (the repulsion's totals).
+cudaError_t launch_pack(const void *K, int dtype, int64_t N, float4 *pos, const float *rho, int nx,
+                        int ny, int nz, int gxp, double lo, double hi, float *rho_out,
+                        float *coords, unsigned long long *zero, int64_t n_zero, int *status,
+                        int sms, cudaStream_t st);
 size_t attraction_smem_bytes(int gxp);
 int attraction_ctas_per_sm(int acc, bool energy, int variant);
 cudaError_t launch_attraction(const AttrArgs &a, int acc, bool energy, int variant, cudaStream_t st);
@@ -201,6 +206,10 @@ int sym_variant_threads(int v);
 size_t repulsion_sym_smem_bytes();
 int repulsion_sym_ctas_per_sm(bool energy, int variant);
 cudaError_t launch_repulsion_sym(const SymArgs &a, bool energy, int variant, cudaStream_t st);
+// Directed repulsion of few samples (repulsion_small.cu) into the symmetric
+// kernel's totals.
+cudaError_t launch_repulsion_small(const float4 *pos, int64_t N, float eps2, bool energy,
+                                   unsigned long long *acc, int sms, cudaStream_t st);
 int energy_blocks(int64_t N);
 cudaError_t launch_combine_energy(const CombineArgs &c, double *out2, cudaStream_t st);
 

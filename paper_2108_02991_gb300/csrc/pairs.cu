@@ -37,8 +37,8 @@ namespace sparkling {
 namespace {
 
 template <typename KT>
-__global__ void pack_positions_kernel(const KT *__restrict__ K, int64_t N, float4 *__restrict__ out,
-                                      int *status)
+__device__ __forceinline__ int pack_positions(const KT *__restrict__ K, int64_t N,
+                                              float4 *__restrict__ out)
 {
     int bad = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
@@ -47,15 +47,14 @@ __global__ void pack_positions_kernel(const KT *__restrict__ K, int64_t N, float
         bad |= !(isfinite(x) && isfinite(y) && isfinite(z));
         out[i] = make_float4(x, y, z, 0.f);
     }
-    if (__syncthreads_or(bad) && threadIdx.x == 0)
-        atomicOr(status, kDevNonFinite);
+    return bad;
 }
 
 // Density rows padded to gxp (multiple of 4) with zeros, and the cell-centre
 // coordinate tables computed in double and rounded once to float.
-__global__ void pack_grid_kernel(const float *__restrict__ rho, int nx, int ny, int nz, int gxp,
-                                 double lo, double hi, float *__restrict__ rho_out,
-                                 float *__restrict__ coords, int *status)
+__device__ __forceinline__ int pack_grid(const float *__restrict__ rho, int nx, int ny, int nz,
+                                         int gxp, double lo, double hi,
+                                         float *__restrict__ rho_out, float *__restrict__ coords)
 {
     const int64_t rows = (int64_t)ny * nz;
     const int64_t total = rows * gxp;
@@ -80,8 +79,43 @@ __global__ void pack_grid_kernel(const float *__restrict__ rho, int nx, int ny, 
         else { q = (int)(e - gxp - ny); n = nz; }
         coords[e] = (q < n) ? (float)(lo + ((double)q + 0.5) * ((hi - lo) / (double)n)) : 0.f;
     }
+    return bad;
+}
+
+__device__ __forceinline__ void flag_bad(int bad, int *status)
+{
     if (__syncthreads_or(bad) && threadIdx.x == 0)
         atomicOr(status, kDevNonFinite);
+}
+
+template <typename KT>
+__global__ void pack_positions_kernel(const KT *__restrict__ K, int64_t N, float4 *__restrict__ out,
+                                      int *status)
+{
+    flag_bad(pack_positions<KT>(K, N, out), status);
+}
+
+__global__ void pack_grid_kernel(const float *__restrict__ rho, int nx, int ny, int nz, int gxp,
+                                 double lo, double hi, float *__restrict__ rho_out,
+                                 float *__restrict__ coords, int *status)
+{
+    flag_bad(pack_grid(rho, nx, ny, nz, gxp, lo, hi, rho_out, coords), status);
+}
+
+// One launch instead of three: samples, density and the cleared totals.
+template <typename KT>
+__global__ void pack_kernel(const KT *__restrict__ K, int64_t N, float4 *__restrict__ pos,
+                            const float *__restrict__ rho, int nx, int ny, int nz, int gxp,
+                            double lo, double hi, float *__restrict__ rho_out,
+                            float *__restrict__ coords, unsigned long long *__restrict__ zero,
+                            int64_t n_zero, int *status)
+{
+    int bad = pack_positions<KT>(K, N, pos);
+    bad |= pack_grid(rho, nx, ny, nz, gxp, lo, hi, rho_out, coords);
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_zero;
+         e += (int64_t)gridDim.x * blockDim.x)
+        zero[e] = 0ull;
+    flag_bad(bad, status);
 }
 
 // Resident CTAs the launch bounds ask for: three at 128 or 256 threads per
@@ -118,40 +152,89 @@ __global__ void __launch_bounds__(NT, min_ctas(NT)) attraction_kernel(const Attr
     }
 }
 
+// Sample i's G = A - R/N (and A, R/N) from its sums, scaled, to the outputs.
+template <typename OT>
+__device__ __forceinline__ void combine_sample(const CombineArgs &c, int64_t i, dacc4 a, double invN,
+                                               double sc)
+{
+    dacc4 r;
+    if (c.r_direct) {
+        r = c.r_direct[i];
+    } else if (c.racc) {
+        r.x = (double)(long long)c.racc[3 * i] / kFixScale;
+        r.y = (double)(long long)c.racc[3 * i + 1] / kFixScale;
+        r.z = (double)(long long)c.racc[3 * i + 2] / kFixScale;
+        r.w = 0.0;
+    } else {
+        r = sum_slots(c.part_r, c.spr, i);
+    }
+    double rx = r.x * invN, ry = r.y * invN, rz = r.z * invN;
+    double gx = a.x - rx, gy = a.y - ry, gz = a.z - rz;
+    if (sc != 1.0) {
+        gx *= sc; gy *= sc; gz *= sc;
+        a.x *= sc; a.y *= sc; a.z *= sc;
+        rx *= sc; ry *= sc; rz *= sc;
+    }
+    OT *G = static_cast<OT *>(c.G);
+    if (G) { G[3 * i] = (OT)gx; G[3 * i + 1] = (OT)gy; G[3 * i + 2] = (OT)gz; }
+    if (c.G64) { c.G64[3 * i] = gx; c.G64[3 * i + 1] = gy; c.G64[3 * i + 2] = gz; }
+    OT *A = static_cast<OT *>(c.A);
+    if (A) { A[3 * i] = (OT)a.x; A[3 * i + 1] = (OT)a.y; A[3 * i + 2] = (OT)a.z; }
+    OT *R = static_cast<OT *>(c.R);
+    if (R) { R[3 * i] = (OT)rx; R[3 * i + 1] = (OT)ry; R[3 * i + 2] = (OT)rz; }
+}
+
 template <typename OT>
 __global__ void combine_kernel(const CombineArgs c)
 {
     const double invN = 1.0 / (double)c.N;
     const double sc = c.scale_dev ? c.scale * c.scale_dev[0] : c.scale;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c.N;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        dacc4 a = c.a_direct ? c.a_direct[i] : sum_slots(c.part_a, c.spa, i);
-        dacc4 r;
-        if (c.r_direct) {
-            r = c.r_direct[i];
-        } else if (c.racc) {
-            r.x = (double)(long long)c.racc[3 * i] / kFixScale;
-            r.y = (double)(long long)c.racc[3 * i + 1] / kFixScale;
-            r.z = (double)(long long)c.racc[3 * i + 2] / kFixScale;
-            r.w = 0.0;
-        } else {
-            r = sum_slots(c.part_r, c.spr, i);
+         i += (int64_t)gridDim.x * blockDim.x)
+        combine_sample<OT>(c, i, c.a_direct ? c.a_direct[i] : sum_slots(c.part_a, c.spa, i), invN, sc);
+}
+
+// Few samples: a tile's attraction is split over up to a whole wave of CTAs
+// (456 slots for one tile), and one thread a sample would add them one after
+// the other (1024 samples: 70 us).  A block takes 32 samples, 8 threads each:
+// thread g adds slots g, g + 8, ..., the eight sums are added in order.
+// 1024 samples: 16 us.
+constexpr int kSlotLanes = 8, kSlotSamples = 32;
+constexpr int64_t kSlotLanesMin = 8;           // slots from which this form is taken
+
+__device__ dacc4 block_sum_slots(const dacc4 *part, const Split &sp, int64_t i, int64_t N)
+{
+    __shared__ dacc4 sums[kSlotLanes][kSlotSamples];
+    const int l = threadIdx.x % kSlotSamples, g = threadIdx.x / kSlotSamples;
+    dacc4 s = make_dacc4(0.0, 0.0, 0.0, 0.0);
+    if (i < N) {
+        const int64_t tile = i / kTile, e = i - tile * kTile;
+        const int64_t n = split_cta_of(sp, (tile + 1) * sp.per_tile - 1) -
+                          split_cta_of(sp, tile * sp.per_tile) + 1;
+#pragma unroll 4
+        for (int64_t j = g; j < n; j += kSlotLanes) {
+            const dacc4 v = part[(tile * sp.slots + j) * kTile + e];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
-        double rx = r.x * invN, ry = r.y * invN, rz = r.z * invN;
-        double gx = a.x - rx, gy = a.y - ry, gz = a.z - rz;
-        if (sc != 1.0) {
-            gx *= sc; gy *= sc; gz *= sc;
-            a.x *= sc; a.y *= sc; a.z *= sc;
-            rx *= sc; ry *= sc; rz *= sc;
-        }
-        OT *G = static_cast<OT *>(c.G);
-        if (G) { G[3 * i] = (OT)gx; G[3 * i + 1] = (OT)gy; G[3 * i + 2] = (OT)gz; }
-        if (c.G64) { c.G64[3 * i] = gx; c.G64[3 * i + 1] = gy; c.G64[3 * i + 2] = gz; }
-        OT *A = static_cast<OT *>(c.A);
-        if (A) { A[3 * i] = (OT)a.x; A[3 * i + 1] = (OT)a.y; A[3 * i + 2] = (OT)a.z; }
-        OT *R = static_cast<OT *>(c.R);
-        if (R) { R[3 * i] = (OT)rx; R[3 * i + 1] = (OT)ry; R[3 * i + 2] = (OT)rz; }
     }
+    sums[g][l] = s;
+    __syncthreads();
+    if (g == 0)
+        for (int k = 1; k < kSlotLanes; ++k) {
+            const dacc4 v = sums[k][l];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+    return s;                                  // complete in the threads with g = 0
+}
+
+template <typename OT>
+__global__ void __launch_bounds__(kSlotLanes * kSlotSamples) combine_few_kernel(const CombineArgs c)
+{
+    const double invN = 1.0 / (double)c.N;
+    const double sc = c.scale_dev ? c.scale * c.scale_dev[0] : c.scale;
+    const int64_t i = (int64_t)blockIdx.x * kSlotSamples + threadIdx.x % kSlotSamples;
+    const dacc4 a = block_sum_slots(c.part_a, c.spa, i, c.N);
+    if (threadIdx.x < kSlotSamples && i < c.N) combine_sample<OT>(c, i, a, invN, sc);
 }
 
 constexpr int kEnergyThreads = 256;
@@ -187,6 +270,24 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_block_kernel(const Comb
                              : c.racc ? (double)(long long)c.racc[i] / kFixScale
                                       : sum_slots(c.part_r, c.spr, i).w;
         }
+    }
+    const double2 s = block_sum2(ea, er);
+    if (threadIdx.x == 0)
+        c.energy_blocks[blockIdx.x] = s;
+}
+
+// The same for few samples: kSlotSamples targets a block, eight threads each.
+__global__ void __launch_bounds__(kEnergyThreads) energy_few_kernel(const CombineArgs c)
+{
+    static_assert(kEnergyThreads == kSlotLanes * kSlotSamples, "block shape");
+    const int64_t i = (int64_t)blockIdx.x * kSlotSamples + threadIdx.x % kSlotSamples;
+    const dacc4 a = block_sum_slots(c.part_a, c.spa, i, c.N);
+    double ea = 0.0, er = 0.0;
+    if (threadIdx.x < kSlotSamples && i < c.N) {
+        ea = a.w;
+        er = c.r_direct ? c.r_direct[i].w
+                        : c.racc ? (double)(long long)c.racc[i] / kFixScale
+                                 : sum_slots(c.part_r, c.spr, i).w;
     }
     const double2 s = block_sum2(ea, er);
     if (threadIdx.x == 0)
@@ -267,6 +368,23 @@ cudaError_t launch_pack_grid(const float *rho, int nx, int ny, int nz, int gxp, 
     return cudaGetLastError();
 }
 
+cudaError_t launch_pack(const void *K, int dtype, int64_t N, float4 *pos, const float *rho, int nx,
+                        int ny, int nz, int gxp, double lo, double hi, float *rho_out,
+                        float *coords, unsigned long long *zero, int64_t n_zero, int *status,
+                        int sms, cudaStream_t st)
+{
+    const int64_t cells = (int64_t)ny * nz * gxp;
+    const int64_t most = N > cells ? (N > n_zero ? N : n_zero) : (cells > n_zero ? cells : n_zero);
+    const int g = grid_for(most, 256, sms);
+    if (dtype == 0)
+        pack_kernel<float><<<g, 256, 0, st>>>(static_cast<const float *>(K), N, pos, rho, nx, ny, nz,
+                                              gxp, lo, hi, rho_out, coords, zero, n_zero, status);
+    else
+        pack_kernel<double><<<g, 256, 0, st>>>(static_cast<const double *>(K), N, pos, rho, nx, ny,
+                                               nz, gxp, lo, hi, rho_out, coords, zero, n_zero, status);
+    return cudaGetLastError();
+}
+
 int attr_variant_threads(int v) { return v == 0 ? 128 : (v == 2 ? 512 : 256); }
 
 size_t attraction_smem_bytes(int)
@@ -296,8 +414,25 @@ cudaError_t launch_attraction(const AttrArgs &a, int acc, bool energy, int varia
                             attraction_smem_bytes(a.gxp), st);
 }
 
+namespace {
+// Samples up to which one block a kSlotSamples samples is launched.
+constexpr int64_t kFewSamples = 1 << 16;
+bool few_samples(const CombineArgs &c)
+{
+    return !c.a_direct && c.spa.slots >= kSlotLanesMin && c.N <= kFewSamples;
+}
+} // namespace
+
 cudaError_t launch_combine(const CombineArgs &c, int out_dtype, int sms, cudaStream_t st)
 {
+    if (few_samples(c)) {
+        const unsigned nb = (unsigned)((c.N + kSlotSamples - 1) / kSlotSamples);
+        if (out_dtype == 0)
+            combine_few_kernel<float><<<nb, kSlotLanes * kSlotSamples, 0, st>>>(c);
+        else
+            combine_few_kernel<double><<<nb, kSlotLanes * kSlotSamples, 0, st>>>(c);
+        return cudaGetLastError();
+    }
     const int g = grid_for(c.N, 256, sms);
     if (out_dtype == 0)
         combine_kernel<float><<<g, 256, 0, st>>>(c);
@@ -306,12 +441,23 @@ cudaError_t launch_combine(const CombineArgs &c, int out_dtype, int sms, cudaStr
     return cudaGetLastError();
 }
 
-int energy_blocks(int64_t N) { return (int)((N + kEnergyBlock - 1) / kEnergyBlock); }
+// Block sums of an energy reduction of N samples, at most.
+int energy_blocks(int64_t N)
+{
+    const int64_t few = ((N < kFewSamples ? N : kFewSamples) + kSlotSamples - 1) / kSlotSamples;
+    const int64_t many = (N + kEnergyBlock - 1) / kEnergyBlock;
+    return (int)(few > many ? few : many);
+}
 
 cudaError_t launch_combine_energy(const CombineArgs &c, double *out2, cudaStream_t st)
 {
-    const int nb = energy_blocks(c.N);
-    energy_block_kernel<<<nb, kEnergyThreads, 0, st>>>(c);
+    const bool few = few_samples(c);
+    const int nb = few ? (int)((c.N + kSlotSamples - 1) / kSlotSamples)
+                       : (int)((c.N + kEnergyBlock - 1) / kEnergyBlock);
+    if (few)
+        energy_few_kernel<<<nb, kEnergyThreads, 0, st>>>(c);
+    else
+        energy_block_kernel<<<nb, kEnergyThreads, 0, st>>>(c);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     energy_final_kernel<<<1, kEnergyThreads, 0, st>>>(c.energy_blocks, nb, c.N, c.eps, out2);

@@ -195,46 +195,50 @@ __global__ void combine_kernel(const CombineArgs c)
 }
 
 // Few samples: a tile's attraction is split over up to a whole wave of CTAs
-// (456 slots for one tile), and one thread a sample would add them one after
-// the other (1024 samples: 70 us).  A block takes 32 samples, 8 threads each:
-// thread g adds slots g, g + 8, ..., the eight sums are added in order.
-// 1024 samples: 16 us.
-constexpr int kSlotLanes = 8, kSlotSamples = 32;
-constexpr int64_t kSlotLanesMin = 8;           // slots from which this form is taken
+// (304 or 456 slots for one tile), and one thread a sample would add them one
+// after the other (1024 samples: 70 us).  A block of 256 threads takes 256 /
+// LANES samples, LANES threads each: thread g adds slots g, g + LANES, ..., and
+// the LANES sums are added in order.  Bound: the FP64 pipe (three adds a slot),
+// so with many slots 32 threads a sample, which spreads 1024 samples over 128
+// SMs (8 threads: 16 us on 32 SMs; the whole gradient call 48 -> 41 us).
+constexpr int kFewThreads = 256;
+constexpr int64_t kFewSlots = 8;               // slots from which this form is taken,
+constexpr int64_t kManySlots = 64;             // and with 32 threads a sample
 
+template <int LANES, bool ENERGY>
 __device__ dacc4 block_sum_slots(const dacc4 *part, const Split &sp, int64_t i, int64_t N)
 {
-    __shared__ dacc4 sums[kSlotLanes][kSlotSamples];
-    const int l = threadIdx.x % kSlotSamples, g = threadIdx.x / kSlotSamples;
+    constexpr int S = kFewThreads / LANES;
+    __shared__ dacc4 sums[LANES][S];
+    const int l = threadIdx.x % S, g = threadIdx.x / S;
     dacc4 s = make_dacc4(0.0, 0.0, 0.0, 0.0);
+    auto add = [](dacc4 &a, const dacc4 &v) {  // the energy alone, or the force alone
+        if (ENERGY) { a.w += v.w; return; }
+        a.x += v.x; a.y += v.y; a.z += v.z;
+    };
     if (i < N) {
         const int64_t tile = i / kTile, e = i - tile * kTile;
         const int64_t n = split_cta_of(sp, (tile + 1) * sp.per_tile - 1) -
                           split_cta_of(sp, tile * sp.per_tile) + 1;
 #pragma unroll 4
-        for (int64_t j = g; j < n; j += kSlotLanes) {
-            const dacc4 v = part[(tile * sp.slots + j) * kTile + e];
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-        }
+        for (int64_t j = g; j < n; j += LANES) add(s, part[(tile * sp.slots + j) * kTile + e]);
     }
     sums[g][l] = s;
     __syncthreads();
     if (g == 0)
-        for (int k = 1; k < kSlotLanes; ++k) {
-            const dacc4 v = sums[k][l];
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-        }
+        for (int k = 1; k < LANES; ++k) add(s, sums[k][l]);
     return s;                                  // complete in the threads with g = 0
 }
 
-template <typename OT>
-__global__ void __launch_bounds__(kSlotLanes * kSlotSamples) combine_few_kernel(const CombineArgs c)
+template <typename OT, int LANES>
+__global__ void __launch_bounds__(kFewThreads) combine_few_kernel(const CombineArgs c)
 {
+    constexpr int S = kFewThreads / LANES;
     const double invN = 1.0 / (double)c.N;
     const double sc = c.scale_dev ? c.scale * c.scale_dev[0] : c.scale;
-    const int64_t i = (int64_t)blockIdx.x * kSlotSamples + threadIdx.x % kSlotSamples;
-    const dacc4 a = block_sum_slots(c.part_a, c.spa, i, c.N);
-    if (threadIdx.x < kSlotSamples && i < c.N) combine_sample<OT>(c, i, a, invN, sc);
+    const int64_t i = (int64_t)blockIdx.x * S + threadIdx.x % S;
+    const dacc4 a = block_sum_slots<LANES, false>(c.part_a, c.spa, i, c.N);
+    if (threadIdx.x < S && i < c.N) combine_sample<OT>(c, i, a, invN, sc);
 }
 
 constexpr int kEnergyThreads = 256;
@@ -276,14 +280,16 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_block_kernel(const Comb
         c.energy_blocks[blockIdx.x] = s;
 }
 
-// The same for few samples: kSlotSamples targets a block, eight threads each.
+// The same for few samples, LANES threads each.
+template <int LANES>
 __global__ void __launch_bounds__(kEnergyThreads) energy_few_kernel(const CombineArgs c)
 {
-    static_assert(kEnergyThreads == kSlotLanes * kSlotSamples, "block shape");
-    const int64_t i = (int64_t)blockIdx.x * kSlotSamples + threadIdx.x % kSlotSamples;
-    const dacc4 a = block_sum_slots(c.part_a, c.spa, i, c.N);
+    static_assert(kEnergyThreads == kFewThreads, "block shape");
+    constexpr int S = kFewThreads / LANES;
+    const int64_t i = (int64_t)blockIdx.x * S + threadIdx.x % S;
+    const dacc4 a = block_sum_slots<LANES, true>(c.part_a, c.spa, i, c.N);
     double ea = 0.0, er = 0.0;
-    if (threadIdx.x < kSlotSamples && i < c.N) {
+    if (threadIdx.x < S && i < c.N) {
         ea = a.w;
         er = c.r_direct ? c.r_direct[i].w
                         : c.racc ? (double)(long long)c.racc[i] / kFixScale
@@ -415,22 +421,33 @@ cudaError_t launch_attraction(const AttrArgs &a, int acc, bool energy, int varia
 }
 
 namespace {
-// Samples up to which one block a kSlotSamples samples is launched.
+// Samples up to which a block of 256 / LANES samples is launched for each.
 constexpr int64_t kFewSamples = 1 << 16;
-bool few_samples(const CombineArgs &c)
+// Threads a sample of the slot sums: 0 (one thread a sample, grid-stride), 8, 32.
+int slot_lanes(const CombineArgs &c)
 {
-    return !c.a_direct && c.spa.slots >= kSlotLanesMin && c.N <= kFewSamples;
+    if (c.a_direct || c.spa.slots < kFewSlots || c.N > kFewSamples) return 0;
+    return c.spa.slots >= kManySlots ? 32 : 8;
+}
+int few_blocks(int64_t N, int lanes)
+{
+    const int64_t s = kFewThreads / lanes;
+    return (int)((N + s - 1) / s);
 }
 } // namespace
 
 cudaError_t launch_combine(const CombineArgs &c, int out_dtype, int sms, cudaStream_t st)
 {
-    if (few_samples(c)) {
-        const unsigned nb = (unsigned)((c.N + kSlotSamples - 1) / kSlotSamples);
-        if (out_dtype == 0)
-            combine_few_kernel<float><<<nb, kSlotLanes * kSlotSamples, 0, st>>>(c);
+    if (const int lanes = slot_lanes(c)) {
+        const int nb = few_blocks(c.N, lanes);
+        if (lanes == 8 && out_dtype == 0)
+            combine_few_kernel<float, 8><<<nb, kFewThreads, 0, st>>>(c);
+        else if (lanes == 8)
+            combine_few_kernel<double, 8><<<nb, kFewThreads, 0, st>>>(c);
+        else if (out_dtype == 0)
+            combine_few_kernel<float, 32><<<nb, kFewThreads, 0, st>>>(c);
         else
-            combine_few_kernel<double><<<nb, kSlotLanes * kSlotSamples, 0, st>>>(c);
+            combine_few_kernel<double, 32><<<nb, kFewThreads, 0, st>>>(c);
         return cudaGetLastError();
     }
     const int g = grid_for(c.N, 256, sms);
@@ -444,18 +461,19 @@ cudaError_t launch_combine(const CombineArgs &c, int out_dtype, int sms, cudaStr
 // Block sums of an energy reduction of N samples, at most.
 int energy_blocks(int64_t N)
 {
-    const int64_t few = ((N < kFewSamples ? N : kFewSamples) + kSlotSamples - 1) / kSlotSamples;
+    const int64_t few = few_blocks(N < kFewSamples ? N : kFewSamples, 32);
     const int64_t many = (N + kEnergyBlock - 1) / kEnergyBlock;
     return (int)(few > many ? few : many);
 }
 
 cudaError_t launch_combine_energy(const CombineArgs &c, double *out2, cudaStream_t st)
 {
-    const bool few = few_samples(c);
-    const int nb = few ? (int)((c.N + kSlotSamples - 1) / kSlotSamples)
-                       : (int)((c.N + kEnergyBlock - 1) / kEnergyBlock);
-    if (few)
-        energy_few_kernel<<<nb, kEnergyThreads, 0, st>>>(c);
+    const int lanes = slot_lanes(c);
+    const int nb = lanes ? few_blocks(c.N, lanes) : (int)((c.N + kEnergyBlock - 1) / kEnergyBlock);
+    if (lanes == 8)
+        energy_few_kernel<8><<<nb, kEnergyThreads, 0, st>>>(c);
+    else if (lanes == 32)
+        energy_few_kernel<32><<<nb, kEnergyThreads, 0, st>>>(c);
     else
         energy_block_kernel<<<nb, kEnergyThreads, 0, st>>>(c);
     cudaError_t e = cudaGetLastError();

@@ -222,6 +222,17 @@ SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, i
                                             const double *g_dev, double scale, void *dK,
                                             int dK_dtype, void *stream);
 
+/* sparkling_energy and its gradient together, for automatic differentiation:
+ * where one pass over the pairs of the attraction gives both (direct sums,
+ * ACC_KAHAN32 or ACC_FP64), also writes dK = dF/dK = (A - R) / N, [N][3] of
+ * double on the device, and sets *wrote = 1; otherwise only the energy is
+ * computed and *wrote = 0 (use sparkling_energy_backward).  Blocks on
+ * `stream`. */
+SPARKLING_API int sparkling_energy_and_grad(sparkling_ctx *ctx, const void *K, int K_dtype,
+                                            int64_t N, const sparkling_grid *grid, int acc,
+                                            double *F_host, double *Fa_host, double *Fr_host,
+                                            double *dK, int *wrote, void *stream);
+
 /* Projection of each of Nc shots of Ns samples onto the constraint set
  * (Sec. II-D, Suppl. Sec. I), in place on K ([Nc*Ns][3], K_dtype), with the
  * dual FISTA iteration in FP64 (or, for FP32 K, in two-float sums of 48 bits,

@@ -30,7 +30,7 @@ REPULSION_DIRECT, REPULSION_MESH = 0, 1
 # Every entry point declared in include/sparkling.h.
 ABI_SYMBOLS = (
     "sparkling_create", "sparkling_destroy", "sparkling_last_error", "sparkling_grad",
-    "sparkling_energy", "sparkling_energy_backward", "sparkling_project", "sparkling_step",
+    "sparkling_energy", "sparkling_energy_backward", "sparkling_energy_and_grad", "sparkling_project", "sparkling_step",
     "sparkling_step_host", "sparkling_status", "sparkling_set_timing", "sparkling_kernel_times",
     "sparkling_launch_count", "sparkling_version", "sparkling_grad_noalloc",
     "sparkling_step_batched", "sparkling_set_autotune", "sparkling_tuning_report",
@@ -113,6 +113,7 @@ def lib() -> ctypes.CDLL:
             "sparkling_grad": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, i, p, p, p], i),
             "sparkling_energy": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, p, p, p], i),
             "sparkling_energy_backward": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, d, p, i, p], i),
+            "sparkling_energy_and_grad": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, p, p, p, p, p], i),
             "sparkling_project": ([p, p, i, i64, i64, ctypes.POINTER(Proj), p, p], i),
             "sparkling_step": ([p, p, i, i64, i64, ctypes.POINTER(Grid), i, d, ctypes.POINTER(Proj), p], i),
             "sparkling_step_host": ([p, p, i, i64, i64, ctypes.POINTER(Grid), p, i, d,
@@ -306,6 +307,19 @@ def sparkling_energy_backward(ctx: Context, K, grid: Grid, g=None, scale: float 
         ctx.handle, _dev_ptr(K, "K"), _dtype_code(K), _rows(K), ctypes.byref(grid), acc,
         _dev_ptr(g, "g"), float(scale), _dev_ptr(dK, "dK"), _dtype_code(dK), _stream(stream)))
     return dK
+
+
+def sparkling_energy_and_grad(ctx: Context, K, grid: Grid, acc: int = ACC_KAHAN32, stream=None):
+    """((F, F^a, F^r), dF/dK as float64 or None): the gradient where one pass
+    gives both (direct sums); blocks on the stream."""
+    import torch
+    F, Fa, Fr, wrote = ctypes.c_double(), ctypes.c_double(), ctypes.c_double(), ctypes.c_int()
+    dK = torch.empty(K.shape, dtype=torch.float64, device=K.device)
+    _check(ctx, lib().sparkling_energy_and_grad(
+        ctx.handle, _dev_ptr(K, "K"), _dtype_code(K), _rows(K), ctypes.byref(grid), acc,
+        ctypes.byref(F), ctypes.byref(Fa), ctypes.byref(Fr), _dev_ptr(dK, "dK"),
+        ctypes.byref(wrote), _stream(stream)))
+    return (F.value, Fa.value, Fr.value), dK if wrote.value else None
 
 
 def sparkling_project(ctx: Context, K, Nc: int, Ns: int, proj: Proj, want_violation: bool = False,

@@ -59,7 +59,7 @@ struct sparkling_ctx {
     int64_t launches = 0;
     // occupancy cache [acc][energy][variant] (the directed repulsion has no
     // plain FP64-accumulate form: it runs with the FP64 fold, rep_acc())
-    int occ_attr[3][2][kAttrVariants] = {};
+    int occ_attr[3][3][kAttrVariants] = {};   // force, energy, both
     int occ_rep[2][2][kRepVariants] = {};
     bool occ_done = false;
     // autotuner: tile shape per (acc, padded row length) for the attraction
@@ -429,7 +429,10 @@ int ensure_occupancy(sparkling_ctx *ctx)
     for (int acc = 0; acc < 3; ++acc)
         for (int e = 0; e < 2; ++e) {
             for (int v = 0; v < kAttrVariants; ++v)
-                ctx->occ_attr[acc][e][v] = attraction_ctas_per_sm(acc, e != 0, v);
+                ctx->occ_attr[acc][e][v] = attraction_ctas_per_sm(acc, e, v);
+            if (acc < 2 && e == 1)
+                for (int v = 0; v < kAttrVariants; ++v)
+                    ctx->occ_attr[acc][2][v] = attraction_ctas_per_sm(acc, 2, v);
             if (acc < 2)
                 for (int v = 0; v < kRepVariants; ++v)
                     ctx->occ_rep[acc][e][v] = repulsion_ctas_per_sm(acc, e != 0, v);
@@ -459,19 +462,21 @@ int attr_choice_of(const sparkling_ctx *ctx, int acc, int gxp)
 }
 
 // Splits of the two pair kernels for the chosen tile shapes.
-void set_splits(sparkling_ctx *ctx, PairPlan &P, int acc, bool energy, int va, int vr)
+void set_splits(sparkling_ctx *ctx, PairPlan &P, int acc, int mode, int va, int vr)
 {
-    const int e = energy ? 1 : 0;
+    const int e = mode;
     const int64_t rows = (int64_t)P.ny * P.nz;
     const int64_t nblocks = (P.N + kSrcBlock - 1) / kSrcBlock;
     if (ctx->occ_attr[acc][e][va] < 1) va = kAttrDefault;   // a pinned shape that cannot be resident
     P.va = va;
     P.vr = vr;
     P.spa = make_split(P.tiles, rows, (int64_t)ctx->sms * ctx->occ_attr[acc][e][va]);
-    P.spr = make_split(P.tiles, nblocks, (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][e][vr]);
+    P.spr = make_split(P.tiles, nblocks,
+                       (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][mode == 1 ? 1 : 0][vr]);
 }
 
-int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, bool energy,
+// mode: the gradient (0), the energy (1), or both (2).
+int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, int mode,
                bool need_g64, PairPlan &P, Carve &cv)
 {
     int s;
@@ -481,7 +486,7 @@ int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, 
     P.gxp = (P.nx + 3) / 4 * 4;
     P.tiles = (N + kTile - 1) / kTile;
     const int va = attr_choice_of(ctx, acc, P.gxp), vr = ctx->rep_choice[rep_acc(acc)];
-    set_splits(ctx, P, acc, energy, va < 0 ? kAttrDefault : va, vr < 0 ? kRepDefault : vr);
+    set_splits(ctx, P, acc, mode, va < 0 ? kAttrDefault : va, vr < 0 ? kRepDefault : vr);
     // Partial buffers big enough for every tile shape and for the tuning
     // trials (which run on a prefix of the tiles with one wave of CTAs).
     int64_t max_ctas = 0;
@@ -499,7 +504,7 @@ int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, 
     P.o_coords = cv.take(((size_t)P.gxp + P.ny + P.nz) * sizeof(float));
     P.o_parta = cv.take((size_t)part_units * kTile * sizeof(dacc4));
     P.o_partr = cv.take((size_t)part_units * kTile * sizeof(dacc4));
-    P.o_racc = cv.take((size_t)N * 3 * sizeof(unsigned long long));
+    P.o_racc = cv.take((size_t)N * (mode == 2 ? 4 : 3) * sizeof(unsigned long long));
     P.o_eblocks = cv.take((size_t)energy_blocks(N) * sizeof(double2));
     P.o_g64 = need_g64 ? cv.take((size_t)N * 3 * sizeof(double)) : 0;
     P.o_adir = ctx->attr_mode == SPARKLING_ATTRACTION_FIELD ? cv.take((size_t)N * sizeof(dacc4)) : 0;
@@ -548,7 +553,7 @@ int tune_pairs(sparkling_ctx *ctx, PairPlan &P, int acc, AttrArgs aa, RepArgs ra
             const int occ = ctx->occ_attr[acc][0][v];
             if (occ < 1) continue;
             aa.sp = make_split(tt, rows, (int64_t)ctx->sms * occ);
-            const double ms = timed([&] { return launch_attraction(aa, acc, false, v, st); });
+            const double ms = timed([&] { return launch_attraction(aa, acc, 0, v, st); });
             const double pairs = (double)std::min<int64_t>(tt * kTile, P.N) * (double)P3;
             const double rate = ms > 0 ? pairs / (ms * 1e-3) : 0.0;
             snprintf(line, sizeof line, "attraction gxp=%d threads=%d: %.4g pairs/s\n", P.gxp,
@@ -692,11 +697,60 @@ int ensure_mesh(sparkling_ctx *ctx, cudaStream_t st)
     return SPARKLING_OK;
 }
 
+// The repulsion sums of the packed samples: into the totals racc (few samples,
+// symmetric kernel), into r_direct (mesh; set here) or into ra.part (directed).
+int run_repulsion(sparkling_ctx *ctx, PairPlan &P, const float4 *pos, const RepArgs &ra, int acc,
+                  bool energy, bool small, unsigned long long *racc, dacc4 *&r_direct,
+                  cudaStream_t st)
+{
+    if (ctx->rep_mode == SPARKLING_REPULSION_MESH) {
+        int s;
+        if ((s = ensure_mesh(ctx, st))) return s;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(st, &cap));
+        r_direct = at<dacc4>(ctx, P.o_rdir);
+        const char *what = "";
+        int nk = 0;
+        LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
+        cudaError_t e = mesh_eval(ctx->mesh, pos, P.N, energy, r_direct, ctx->d_status, ctx->sms, st,
+                                  &what, &nk, cap != cudaStreamCaptureStatusNone);
+        if (e == cudaErrorStreamCaptureUnsupported)
+            return fail(ctx, SPARKLING_E_INVAL,
+                        "the fast repulsion's buffers for N = %lld are allocated by a first call "
+                        "of that size outside stream capture", (long long)P.N);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            return fail(ctx, SPARKLING_E_NOMEM, "fast repulsion: %s allocation failed", what);
+        }
+        if (e != cudaSuccess) return cuda_fail(ctx, e, what);
+        ls.done(nk);
+        return SPARKLING_OK;
+    }
+    LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
+    if (small) {
+        CK(launch_repulsion_small(pos, P.N, ra.eps2, energy, racc, ctx->sms, st));
+    } else if (ctx->rep_symmetric) {
+        // every unordered pair once, exact fixed-point totals
+        SymArgs sa{};
+        sa.pos = pos; sa.N = P.N; sa.tiles = P.tiles;
+        const int sv = ctx->sym_choice < 0 ? kSymDefault : ctx->sym_choice;
+        sa.ctas = (int64_t)ctx->sms * ctx->occ_sym[energy ? 1 : 0][sv];
+        sa.acc = racc; sa.status = ctx->d_status; sa.eps2 = ra.eps2;
+        CK(launch_repulsion_sym(sa, energy, sv, st));
+    } else {
+        CK(launch_repulsion(ra, rep_acc(acc), energy, P.vr, st));
+    }
+    ls.done();
+    return SPARKLING_OK;
+}
+
 // pack -> (autotune) -> attraction -> repulsion -> combine (gradient) or
 // energy reduction.  In field mode the attraction is the interpolated node
 // field.
+// mode 0: gradient; 1: energy; 2: both, the attraction's from one pass (the
+// repulsion, at most as many pairs, takes one for each).
 int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_grid *g, int acc,
-              bool energy, PairPlan &P, void *G, int G_dtype, void *A, void *R, bool g64,
+              int mode, PairPlan &P, void *G, int G_dtype, void *A, void *R, bool g64,
               cudaStream_t st, double scale = 1.0, const double *scale_dev = nullptr)
 {
     float4 *pos = at<float4>(ctx, P.o_pos);
@@ -713,7 +767,7 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     const bool small = !mesh_mode && P.N <= kSmallRepulsion && !ctx->pin_sym;
     // fixed-point totals of the repulsion, cleared by the pack
     const bool totals = small || (!mesh_mode && ctx->rep_symmetric);
-    const int64_t n_totals = totals ? P.N * (energy ? 1 : 3) : 0;
+    const int64_t n_totals = totals ? P.N * (mode == 2 ? 4 : mode == 1 ? 1 : 3) : 0;
     {
         LaunchScope ls(ctx, SPARKLING_KERNEL_PACK, st);
         CK(launch_pack(K, K_dtype, P.N, pos, g->rho, P.nx, P.ny, P.nz, P.gxp, g->lo, g->hi, rho,
@@ -744,7 +798,7 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
                                at<unsigned long long>(ctx, P.o_racc), st);
             if (s) return s;
             const int va = attr_choice_of(ctx, acc, P.gxp), vr = ctx->rep_choice[rep_acc(acc)];
-            set_splits(ctx, P, acc, energy, va < 0 ? kAttrDefault : va, vr < 0 ? kRepDefault : vr);
+            set_splits(ctx, P, acc, mode, va < 0 ? kAttrDefault : va, vr < 0 ? kRepDefault : vr);
             if (need_s)      // the trials added into the totals
                 CK(cudaMemsetAsync(at<unsigned long long>(ctx, P.o_racc), 0,
                                    (size_t)n_totals * sizeof(unsigned long long), st));
@@ -759,65 +813,31 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
             CK(launch_interp(pos, P.N, ctx->field, P.nx, P.ny, P.nz, g->lo, g->hi, a_direct,
                              ctx->sms, st));
         else
-            CK(launch_attraction(aa, acc, energy, P.va, st));
-        ls.done();
-    }
-    unsigned long long *racc = nullptr;
-    dacc4 *r_direct = nullptr;
-    if (mesh_mode) {
-        int s;
-        if ((s = ensure_mesh(ctx, st))) return s;
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(cudaStreamIsCapturing(st, &cap));
-        r_direct = at<dacc4>(ctx, P.o_rdir);
-        const char *what = "";
-        int nk = 0;
-        LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
-        cudaError_t e = mesh_eval(ctx->mesh, pos, P.N, energy, r_direct, ctx->d_status, ctx->sms, st,
-                                  &what, &nk, cap != cudaStreamCaptureStatusNone);
-        if (e == cudaErrorStreamCaptureUnsupported)
-            return fail(ctx, SPARKLING_E_INVAL,
-                        "the fast repulsion's buffers for N = %lld are allocated by a first call "
-                        "of that size outside stream capture", (long long)P.N);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            return fail(ctx, SPARKLING_E_NOMEM, "fast repulsion: %s allocation failed", what);
-        }
-        if (e != cudaSuccess) return cuda_fail(ctx, e, what);
-        ls.done(nk);
-    } else if (small) {
-        racc = at<unsigned long long>(ctx, P.o_racc);
-        LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
-        CK(launch_repulsion_small(pos, P.N, ra.eps2, energy, racc, ctx->sms, st));
-        ls.done();
-    } else if (ctx->rep_symmetric) {
-        // every unordered pair once, exact fixed-point totals
-        racc = at<unsigned long long>(ctx, P.o_racc);
-        SymArgs sa{};
-        sa.pos = pos; sa.N = P.N; sa.tiles = P.tiles;
-        const int sv = ctx->sym_choice < 0 ? kSymDefault : ctx->sym_choice;
-        sa.ctas = (int64_t)ctx->sms * ctx->occ_sym[energy ? 1 : 0][sv];
-        sa.acc = racc; sa.status = ctx->d_status; sa.eps2 = ra.eps2;
-        LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
-        CK(launch_repulsion_sym(sa, energy, sv, st));
-        ls.done();
-    } else {
-        LaunchScope ls(ctx, SPARKLING_KERNEL_REPULSION, st);
-        CK(launch_repulsion(ra, rep_acc(acc), energy, P.vr, st));
+            CK(launch_attraction(aa, acc, mode, P.va, st));
         ls.done();
     }
     CombineArgs cb{};
     cb.N = P.N; cb.part_a = aa.part; cb.part_r = ra.part; cb.spa = P.spa; cb.spr = P.spr;
     cb.G = G; cb.A = A; cb.R = R;
     cb.G64 = g64 ? at<double>(ctx, P.o_g64) : nullptr;
-    cb.racc = racc;
     cb.a_direct = a_direct;
-    cb.r_direct = r_direct;
     cb.scale = scale;
     cb.scale_dev = scale_dev;
     cb.eps = ctx->eps;
     cb.energy_blocks = at<double2>(ctx, P.o_eblocks);
-    {
+    // the repulsion's force sums, then (mode 2) or instead (mode 1) its energy sums
+    for (int energy = mode == 1 ? 1 : 0; energy <= (mode == 0 ? 0 : 1); ++energy) {
+        int s;
+        if (mode == 2 && energy)
+            cb.spr = make_split(P.tiles, (P.N + kSrcBlock - 1) / kSrcBlock,
+                                (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][1][P.vr]);
+        ra.sp = cb.spr;
+        unsigned long long *racc = nullptr;
+        if (totals) racc = at<unsigned long long>(ctx, P.o_racc) + (mode == 2 && energy ? 3 * P.N : 0);
+        dacc4 *r_direct = nullptr;
+        if ((s = run_repulsion(ctx, P, pos, ra, acc, energy != 0, small, racc, r_direct, st))) return s;
+        cb.racc = racc;
+        cb.r_direct = r_direct;
         LaunchScope ls(ctx, SPARKLING_KERNEL_COMBINE, st);
         if (energy) {
             CK(launch_combine_energy(cb, ctx->d_small, st));
@@ -1333,9 +1353,9 @@ SPARKLING_API int sparkling_grad(sparkling_ctx *ctx, const void *K, int K_dtype,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, false, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, 0, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    return run_pairs(ctx, K, K_dtype, grid, acc, false, P, G, G_dtype, A, R, false, st);
+    return run_pairs(ctx, K, K_dtype, grid, acc, 0, P, G, G_dtype, A, R, false, st);
 }
 
 SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, int K_dtype,
@@ -1355,9 +1375,9 @@ SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, i
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, false, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, 0, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    return run_pairs(ctx, K, K_dtype, grid, acc, false, P, dK, dK_dtype, nullptr, nullptr, false, st,
+    return run_pairs(ctx, K, K_dtype, grid, acc, 0, P, dK, dK_dtype, nullptr, nullptr, false, st,
                      scale / (double)N, g_dev);
 }
 
@@ -1373,9 +1393,9 @@ SPARKLING_API int sparkling_energy(sparkling_ctx *ctx, const void *K, int K_dtyp
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, true, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, 1, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, true, P, nullptr, 0, nullptr, nullptr, false, st)))
+    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 1, P, nullptr, 0, nullptr, nullptr, false, st)))
         return s;
     double h[2];
     CK(cudaMemcpyAsync(h, ctx->d_small, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1383,6 +1403,40 @@ SPARKLING_API int sparkling_energy(sparkling_ctx *ctx, const void *K, int K_dtyp
     if (Fa_host) *Fa_host = h[0];
     if (Fr_host) *Fr_host = h[1];
     if (F_host) *F_host = h[0] - h[1];
+    return SPARKLING_OK;
+}
+
+SPARKLING_API int sparkling_energy_and_grad(sparkling_ctx *ctx, const void *K, int K_dtype,
+                                            int64_t N, const sparkling_grid *grid, int acc,
+                                            double *F_host, double *Fa_host, double *Fr_host,
+                                            double *dK, int *wrote, void *stream)
+{
+    int s;
+    if (wrote) *wrote = 0;
+    if ((s = common_checks(ctx, K, K_dtype, N, grid, acc))) return s;
+    if (!dK || !wrote) return fail(ctx, SPARKLING_E_INVAL, "dK and wrote are required");
+    // one pass pays where it spares a second attraction sum of every pair
+    if (ctx->attr_mode != SPARKLING_ATTRACTION_DIRECT || ctx->rep_mode != SPARKLING_REPULSION_DIRECT ||
+        acc == SPARKLING_ACC_FP64_PAIR)
+        return sparkling_energy(ctx, K, K_dtype, N, grid, acc, F_host, Fa_host, Fr_host, stream);
+    if ((s = lazy_init(ctx))) return s;
+    if (!is_device_ptr(K) || !is_device_ptr(dK) || !is_device_ptr(grid->rho))
+        return fail(ctx, SPARKLING_E_INVAL, "K, dK and grid->rho must be device memory");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    PairPlan P;
+    Carve cv;
+    if ((s = plan_pairs(ctx, N, grid, acc, 2, false, P, cv))) return s;
+    if ((s = ensure_ws(ctx, P.end))) return s;
+    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 2, P, dK, SPARKLING_F64, nullptr, nullptr, false, st,
+                       1.0 / (double)N)))
+        return s;
+    double h[2];
+    CK(cudaMemcpyAsync(h, ctx->d_small, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    if ((s = read_status(ctx, st))) return s;
+    if (Fa_host) *Fa_host = h[0];
+    if (Fr_host) *Fr_host = h[1];
+    if (F_host) *F_host = h[0] - h[1];
+    *wrote = 1;
     return SPARKLING_OK;
 }
 
@@ -1441,13 +1495,13 @@ SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64
     }
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, false, true, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, 0, true, P, cv))) return s;
     ProjPlan L;
     if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     if ((s = ensure_ws(ctx, cv.off))) return s;
     // the whole device work of the step, timed as one scope when timing is on
     StepScope whole(ctx, st);
-    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, false, P, nullptr, K_dtype, nullptr, nullptr, true,
+    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 0, P, nullptr, K_dtype, nullptr, nullptr, true,
                        st)))
         return s;
     if ((s = run_project(ctx, K, K_dtype, Nc, Ns, proj, at<double>(ctx, P.o_g64), eta, L, false, st)))
@@ -1497,7 +1551,7 @@ int run_optimize(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t N
     PairPlan P;
     Carve cv;
     int s;
-    if ((s = plan_pairs(ctx, N, grid, acc, false, true, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, 0, true, P, cv))) return s;
     ProjPlan L;
     if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     const size_t o_kp = cv.take((size_t)n3 * sizeof(double));
@@ -1507,7 +1561,7 @@ int run_optimize(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t N
     const double *G64 = at<double>(ctx, P.o_g64);
     double step = sc->eta;
     for (int t = 0; t < sc->n_git; ++t) {
-        if ((s = run_pairs(ctx, K, K_dtype, grid, acc, false, P, nullptr, K_dtype, nullptr, nullptr,
+        if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 0, P, nullptr, K_dtype, nullptr, nullptr,
                            true, st)))
             return s;
         const bool bb = t >= sc->n_fixed && t > 0;

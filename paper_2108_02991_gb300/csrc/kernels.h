@@ -187,9 +187,10 @@ cudaError_t launch_pack(const void *K, int dtype, int64_t N, float4 *pos, const 
                         int ny, int nz, int gxp, double lo, double hi, float *rho_out,
                         float *coords, unsigned long long *zero, int64_t n_zero, int *status,
                         int sms, cudaStream_t st);
-size_t attraction_smem_bytes(int gxp);
-int attraction_ctas_per_sm(int acc, bool energy, int variant);
-cudaError_t launch_attraction(const AttrArgs &a, int acc, bool energy, int variant, cudaStream_t st);
+// mode 0: force, 1: energy, 2: both (acc 0 and 1 only).
+size_t attraction_smem_bytes(int mode);
+int attraction_ctas_per_sm(int acc, int mode, int variant);
+cudaError_t launch_attraction(const AttrArgs &a, int acc, int mode, int variant, cudaStream_t st);
 size_t repulsion_smem_bytes();
 int repulsion_ctas_per_sm(int acc, bool energy, int variant);
 cudaError_t launch_repulsion(const RepArgs &a, int acc, bool energy, int variant, cudaStream_t st);

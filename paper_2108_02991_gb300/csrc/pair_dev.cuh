@@ -83,6 +83,7 @@ template <int ACC> struct RowSum { typedef float type; };
 template <> struct RowSum<2> { typedef double type; };
 
 constexpr int kAccBytes = kTile * 3 * 8;   // 24 KB per CTA: 3 values x 8 bytes per target
+constexpr int acc_bytes(int mode) { return mode == 2 ? kTile * 4 * 8 : kAccBytes; }
 
 // NR grid rows (1 or 2) against the thread's T targets.  The rows share the
 // x coordinates, so one dx = kx - x_q feeds NR pairs.  x_q is rebuilt as
@@ -91,13 +92,17 @@ constexpr int kAccBytes = kTile * 3 * 8;   // 24 KB per CTA: 3 values x 8 bytes 
 // are added into the stage accumulators st[t][0..NV).  AT is the type the
 // pair terms are summed in: float (row sums in FP32), or double (every pair
 // term converted and added in FP64: the plain FP64-accumulate form).
-template <bool ENERGY, int NR, int T, typename AT>
+// MODE: the force (0), the energy (1), or both from the same reciprocal square
+// roots (2; the energy is the fourth value).
+template <int MODE, int NR, int T, typename AT>
 __device__ __forceinline__ void attr_rows(const float *rows, int gxp, const float *kxp,
                                           const float *ky, const float *kz, const float *yr,
-                                          const float *zr, float h, float eps2, AT (*st)[3])
+                                          const float *zr, float h, float eps2,
+                                          AT (*st)[MODE == 2 ? 4 : 3])
 {
+    constexpr bool ENERGY = MODE == 1;
     float s2[NR][T];
-    AT sw[NR][T], sx[T];
+    AT sw[NR][T], sx[T], se[NR][T];
 #pragma unroll
     for (int t = 0; t < T; ++t) {
 #pragma unroll
@@ -105,6 +110,7 @@ __device__ __forceinline__ void attr_rows(const float *rows, int gxp, const floa
             const float dy = ky[t] - yr[r], dz = kz[t] - zr[r];
             s2[r][t] = fmaf(dy, dy, fmaf(dz, dz, eps2));
             sw[r][t] = 0.f;
+            if (MODE == 2) se[r][t] = 0.f;
         }
         sx[t] = 0.f;
     }
@@ -136,6 +142,7 @@ __device__ __forceinline__ void attr_rows(const float *rows, int gxp, const floa
                     } else {
                         sw[r][t] += (AT)wt;
                         sx[t] = fma_t((AT)wt, (AT)dx[j], sx[t]);
+                        if (MODE == 2) se[r][t] = fma_t((AT)wt, (AT)r2, se[r][t]);
                     }
                 }
             }
@@ -153,18 +160,20 @@ __device__ __forceinline__ void attr_rows(const float *rows, int gxp, const floa
             for (int r = 0; r < NR; ++r) {
                 st[t][1] = fma_t((AT)(ky[t] - yr[r]), sw[r][t], st[t][1]);
                 st[t][2] = fma_t((AT)(kz[t] - zr[r]), sw[r][t], st[t][2]);
+                if (MODE == 2) st[t][MODE == 2 ? 3 : 0] += se[r][t];
             }
         }
     }
 }
 
-template <int ACC, bool ENERGY, int NT>
+template <int ACC, int MODE, int NT>
 __device__ bool attraction_segment(const AttrArgs &a, int64_t tile, int64_t r0, int64_t r1,
                                    int slot, float *stage, uint64_t *bars, void *accbase,
                                    uint32_t &consumed)
 {
+    constexpr bool ENERGY = MODE == 1;
     constexpr int T = kTile / NT;
-    constexpr int NV = ENERGY ? 1 : 3;
+    constexpr int NV = MODE == 2 ? 4 : ENERGY ? 1 : 3;
     const int tid = threadIdx.x;
     float kxp[T], ky[T], kz[T];
 #pragma unroll
@@ -208,9 +217,12 @@ __device__ bool attraction_segment(const AttrArgs &a, int64_t tile, int64_t r0, 
         const int nrows = (int)((rs + R < r1 ? rs + R : r1) - rs);
         int iy = (int)(rs % a.ny), iz = (int)(rs / a.ny);
         typedef typename RowSum<ACC>::type AT;
-        AT st[T][3];
+        AT st[T][MODE == 2 ? 4 : 3];
 #pragma unroll
-        for (int t = 0; t < T; ++t) st[t][0] = st[t][1] = st[t][2] = (AT)0;
+        for (int t = 0; t < T; ++t) {
+            st[t][0] = st[t][1] = st[t][2] = (AT)0;
+            if (MODE == 2) st[t][MODE == 2 ? 3 : 0] = (AT)0;
+        }
         int rr = 0;
         for (; rr + 1 < nrows; rr += 2) {
             float yr[2], zr[2];
@@ -218,11 +230,11 @@ __device__ bool attraction_segment(const AttrArgs &a, int64_t tile, int64_t r0, 
             if (++iy == a.ny) { iy = 0; ++iz; }
             yr[1] = ys[iy]; zr[1] = zs[iz];
             if (++iy == a.ny) { iy = 0; ++iz; }
-            attr_rows<ENERGY, 2, T, AT>(buf + rr * gxp, gxp, kxp, ky, kz, yr, zr, a.hx, a.eps2, st);
+            attr_rows<MODE, 2, T, AT>(buf + rr * gxp, gxp, kxp, ky, kz, yr, zr, a.hx, a.eps2, st);
         }
         if (rr < nrows) {
             float yr[1] = {ys[iy]}, zr[1] = {zs[iz]};
-            attr_rows<ENERGY, 1, T, AT>(buf + rr * gxp, gxp, kxp, ky, kz, yr, zr, a.hx, a.eps2, st);
+            attr_rows<MODE, 1, T, AT>(buf + rr * gxp, gxp, kxp, ky, kz, yr, zr, a.hx, a.eps2, st);
         }
 #pragma unroll
         for (int t = 0; t < T; ++t)
@@ -240,8 +252,9 @@ __device__ bool attraction_segment(const AttrArgs &a, int64_t tile, int64_t r0, 
         const int l = t * NT + tid;
         if (tile * kTile + l < a.N) {
             dacc4 v = ENERGY ? make_dacc4(0.0, 0.0, 0.0, acc.value(t))
-                             : make_dacc4(acc.value(3 * t), acc.value(3 * t + 1),
-                                          acc.value(3 * t + 2), 0.0);
+                             : make_dacc4(acc.value(NV * t), acc.value(NV * t + 1),
+                                          acc.value(NV * t + 2),
+                                          MODE == 2 ? acc.value(NV * t + 3) : 0.0);
             a.part[(tile * a.sp.slots + slot) * kTile + l] = v;
         }
     }

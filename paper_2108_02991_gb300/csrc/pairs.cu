@@ -123,12 +123,14 @@ __global__ void pack_kernel(const KT *__restrict__ K, int64_t N, float4 *__restr
 // (registers <= 64).
 constexpr int min_ctas(int nt) { return nt >= 512 ? 2 : 3; }
 
-template <int ACC, bool ENERGY, int NT>
+// MODE 0: force, 1: energy, 2: both.
+template <int ACC, int MODE, int NT>
 __global__ void __launch_bounds__(NT, min_ctas(NT)) attraction_kernel(const AttrArgs a)
 {
+    constexpr int kAcc = MODE == 2 ? kTile * 4 * 8 : kAccBytes;
     extern __shared__ __align__(128) float smem[];
-    void *accbase = smem;                                     // kAccBytes
-    float *stage = smem + kAccBytes / sizeof(float);          // kStages * kStageFloats
+    void *accbase = smem;                                     // kAcc bytes
+    float *stage = smem + kAcc / sizeof(float);               // kStages * kStageFloats
     uint64_t *bars = reinterpret_cast<uint64_t *>(stage + kStages * kStageFloats);
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s)
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(NT, min_ctas(NT)) attraction_kernel(const Attr
         const int64_t r0 = u - tile * rows;
         const int64_t r1 = rows < r0 + (uend - u) ? rows : r0 + (uend - u);
         const int slot = (int)(blockIdx.x - split_cta_of(a.sp, tile * rows));
-        if (!attraction_segment<ACC, ENERGY, NT>(a, tile, r0, r1, slot, stage, bars, accbase,
+        if (!attraction_segment<ACC, MODE, NT>(a, tile, r0, r1, slot, stage, bars, accbase,
                                              consumed))
             return;
         u += r1 - r0;
@@ -324,23 +326,25 @@ cudaError_t set_smem(K kernel, size_t bytes)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <int ACC, bool E, int NT>
-void *attraction_fn() { return reinterpret_cast<void *>(attraction_kernel<ACC, E, NT>); }
+template <int ACC, int MODE, int NT>
+void *attraction_fn() { return reinterpret_cast<void *>(attraction_kernel<ACC, MODE, NT>); }
 
+// The plain FP64-accumulate form (acc 2) has no MODE 2.
 template <int NT>
-void *pick_attraction_nt(int acc, bool energy)
+void *pick_attraction_nt(int acc, int mode)
 {
-    if (acc == 0) return energy ? attraction_fn<0, true, NT>() : attraction_fn<0, false, NT>();
-    if (acc == 2) return energy ? attraction_fn<2, true, NT>() : attraction_fn<2, false, NT>();
-    return energy ? attraction_fn<1, true, NT>() : attraction_fn<1, false, NT>();
+    if (acc == 2) return mode == 1 ? attraction_fn<2, 1, NT>() : attraction_fn<2, 0, NT>();
+    if (mode == 2) return acc == 0 ? attraction_fn<0, 2, NT>() : attraction_fn<1, 2, NT>();
+    if (acc == 0) return mode == 1 ? attraction_fn<0, 1, NT>() : attraction_fn<0, 0, NT>();
+    return mode == 1 ? attraction_fn<1, 1, NT>() : attraction_fn<1, 0, NT>();
 }
 
-void *pick_attraction(int acc, bool energy, int variant)
+void *pick_attraction(int acc, int mode, int variant)
 {
     switch (variant) {
-    case 0: return pick_attraction_nt<128>(acc, energy);
-    case 2: return pick_attraction_nt<512>(acc, energy);
-    default: return pick_attraction_nt<256>(acc, energy);
+    case 0: return pick_attraction_nt<128>(acc, mode);
+    case 2: return pick_attraction_nt<512>(acc, mode);
+    default: return pick_attraction_nt<256>(acc, mode);
     }
 }
 
@@ -393,16 +397,16 @@ cudaError_t launch_pack(const void *K, int dtype, int64_t N, float4 *pos, const 
 
 int attr_variant_threads(int v) { return v == 0 ? 128 : (v == 2 ? 512 : 256); }
 
-size_t attraction_smem_bytes(int)
+size_t attraction_smem_bytes(int mode)
 {
-    return (size_t)kAccBytes + (size_t)kStages * kStageFloats * sizeof(float) +
+    return (size_t)acc_bytes(mode) + (size_t)kStages * kStageFloats * sizeof(float) +
            kStages * sizeof(uint64_t);
 }
 
-int attraction_ctas_per_sm(int acc, bool energy, int variant)
+int attraction_ctas_per_sm(int acc, int mode, int variant)
 {
-    void *fn = pick_attraction(acc, energy, variant);
-    const size_t smem = attraction_smem_bytes(0);
+    void *fn = pick_attraction(acc, mode, variant);
+    const size_t smem = attraction_smem_bytes(mode);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;
     int n = 0;
@@ -412,12 +416,12 @@ int attraction_ctas_per_sm(int acc, bool energy, int variant)
     return n;
 }
 
-cudaError_t launch_attraction(const AttrArgs &a, int acc, bool energy, int variant, cudaStream_t st)
+cudaError_t launch_attraction(const AttrArgs &a, int acc, int mode, int variant, cudaStream_t st)
 {
-    void *fn = pick_attraction(acc, energy, variant);
+    void *fn = pick_attraction(acc, mode, variant);
     void *args[] = {const_cast<AttrArgs *>(&a)};
     return cudaLaunchKernel(fn, dim3((unsigned)a.sp.ctas), dim3(attr_variant_threads(variant)), args,
-                            attraction_smem_bytes(a.gxp), st);
+                            attraction_smem_bytes(mode), st);
 }
 
 namespace {

@@ -896,7 +896,7 @@ int plan_project(sparkling_ctx *ctx, int K_dtype, int64_t Nc, int64_t Ns, const 
     const int ns = (int)Ns;
     if (project_reg_applies(K_dtype, ns, pr->alpha, pr->beta, pr->box, pr->tol, pr->pin,
                             pr->pin_index, pr->n_iter)) {
-        L.reg = project_reg_shape(K_dtype, Nc, ns, ctx->sms);
+        L.reg = project_reg_shape(K_dtype, Nc, ns, ctx->sms, true);
         return SPARKLING_OK;
     }
     const int occ = project_ctas_per_sm(K_dtype, ns);
@@ -1754,7 +1754,7 @@ SPARKLING_API int sparkling_step_batched(sparkling_ctx *ctx, int32_t B, const in
         b.one_launch = one_launch;
         b.sym = ctx->rep_symmetric && !one_launch;
         b.split_proj = split_proj;
-        b.proj_shape = project_reg_shape(K_dtype, off[B] / Ns, Ns, ctx->sms);
+        b.proj_shape = project_reg_shape(K_dtype, off[B] / Ns, Ns, ctx->sms, false);
         build_work_list(b, off, grids, ctas, ctx->items_per_cta, b.sym, b.one_launch, !split_proj);
         b.roles = one_launch;
         if (b.roles) split_work_list(b);

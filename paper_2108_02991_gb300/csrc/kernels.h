@@ -285,10 +285,11 @@ cudaError_t launch_project(const ProjArgs &p, int dtype, int grid, cudaStream_t 
 // or ctas = 0 where it does not apply.
 struct RegShape {
     int per_thread = 0, ctas = 0, threads = 0;
+    int own = 0, halo = 0;       // samples a CTA owns and a neighbour's it computes too (halo > 0)
 };
 bool project_reg_applies(int dtype, int Ns, double alpha, double beta, double box, double tol,
                          const double *pin, int pin_index, int n_iter);
-RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms);
+RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms, bool halos);
 // Violations of the result are max-reduced into p.viol when set (a second launch).
 cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, int sms,
                                cudaStream_t st);

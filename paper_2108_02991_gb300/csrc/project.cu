@@ -81,56 +81,141 @@ __global__ void __launch_bounds__(kProjMaxThreads) project_kernel(const ProjArgs
 constexpr __host__ __device__ int reg_max_threads(int M) { return M == 1 ? 768 : 512; }
 constexpr int kRegMaxCtas = 8;                 // portable cluster size
 
+// How the CTAs of one shot meet.
+constexpr int kAlone = 0;        // one CTA
+constexpr int kMeet = 1;         // edges through distributed shared memory, two cluster barriers an iteration
+// A CTA also computes the samples of a halo of its neighbours, whose edge
+// spoils two samples an iteration, and the halos' state is copied from their
+// owners every (halo - 2) / 2 iterations: for shots that leave the GPU idle,
+// where a cluster barrier (~0.5 us) in every iteration would cost as much as
+// the iteration.
+constexpr int kHalo = 2;
+constexpr int kMaxHalo = 32;
+
 // The slots and neighbours of the calling warp; zeroed, and every CTA of the
 // cluster running, on return.
-template <class R, int M, bool CL> struct RegEdges {
+template <class R, int M, int CL> struct RegEdges {
+    struct Shared {
+        EdgeSlot<R> slots[reg_max_threads(M) / 32];
+        R band[CL == kHalo ? 2 : 1][CL == kHalo ? 12 : 1][CL == kHalo ? kMaxHalo : 1];
+    };
+    Shared *sh;
     EdgeSlot<R> *mine, *to_right = nullptr, *to_left = nullptr;
     bool first, last;
-    int C, rank;
+    int C, rank, own, halo;
 
-    __device__ RegEdges(EdgeSlot<R> *slots)
+    __device__ RegEdges(Shared *s, const RegShape &shape) : sh(s), own(shape.own), halo(shape.halo)
     {
         namespace cg = cooperative_groups;
         const cg::cluster_group cl = cg::this_cluster();
         C = CL ? (int)cl.num_blocks() : 1;
         rank = CL ? (int)cl.block_rank() : 0;
         const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-        first = rank == 0 && warp == 0;
-        last = rank == C - 1 && warp == warps - 1;
-        mine = &slots[warp];
-        if (warp < warps - 1) to_right = &slots[warp + 1];
-        else if (CL && !last) to_right = cl.map_shared_rank(&slots[0], rank + 1);
-        if (warp > 0) to_left = &slots[warp - 1];
-        else if (CL && !first) to_left = cl.map_shared_rank(&slots[warps - 1], rank - 1);
+        first = (CL != kMeet || rank == 0) && warp == 0;
+        last = (CL != kMeet || rank == C - 1) && warp == warps - 1;
+        mine = &s->slots[warp];
+        if (warp < warps - 1) to_right = &s->slots[warp + 1];
+        else if (CL == kMeet && !last) to_right = cl.map_shared_rank(&s->slots[0], rank + 1);
+        if (warp > 0) to_left = &s->slots[warp - 1];
+        else if (CL == kMeet && !first) to_left = cl.map_shared_rank(&s->slots[warps - 1], rank - 1);
         for (int q = threadIdx.x; q < warps * kSlotWords; q += blockDim.x)
-            reinterpret_cast<double *>(slots)[q] = 0.0;
-        sync();
+            reinterpret_cast<double *>(s->slots)[q] = 0.0;
+        cluster_sync();
     }
-    __device__ __forceinline__ static void sync()
+    __device__ __forceinline__ static void cta_sync()
     {
-        if (CL) cooperative_groups::this_cluster().sync();
-        else if (blockDim.x == 32) __syncwarp();
+        if (blockDim.x == 32) __syncwarp();
         else __syncthreads();
     }
-    __device__ int first_sample() const { return (rank * (int)blockDim.x + (int)threadIdx.x) * M; }
+    __device__ __forceinline__ static void cluster_sync()
+    {
+        if (CL) cooperative_groups::this_cluster().sync();
+        else cta_sync();
+    }
+    // First sample of the thread; kHalo: the CTA owns [rank * own, (rank + 1) * own)
+    // and begins `halo` before them.
+    __device__ int first_sample() const
+    {
+        if (CL == kHalo) return (rank ? rank * own - halo : 0) + (int)threadIdx.x * M;
+        return (rank * (int)blockDim.x + (int)threadIdx.x) * M;
+    }
+    __device__ __forceinline__ bool owns(int m) const
+    {
+        return CL != kHalo || (m >= rank * own && m < (rank + 1) * own);
+    }
+
+    // Every (halo - 2) / 2 iterations: the owners' state of the halos' samples.
+    // (Before the first one, too: no CTA may store its result over samples that a
+    // neighbour has still to load for its halo.)
+    __device__ __forceinline__ void refresh(int it, int m0, R (*y1)[3], R (*y2)[3], R (*w1)[3],
+                                            R (*w2)[3])
+    {
+        if (CL != kHalo || (it + 1) % ((halo - 2) / 2) != 0) return;
+        namespace cg = cooperative_groups;
+        const cg::cluster_group cl = cg::this_cluster();
+        const int lo = rank * own, hi = lo + own;
+        // the samples that a neighbour's halo holds: band 0 our first ones, band 1 our last
+#pragma unroll
+        for (int j = 0; j < M; ++j) {
+            const int m = m0 + j;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int i = e == 0 ? m - lo : m - (hi - halo);
+                if (m >= lo && m < hi && i >= 0 && i < halo)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        sh->band[e][c][i] = y1[j][c];
+                        sh->band[e][3 + c][i] = y2[j][c];
+                        sh->band[e][6 + c][i] = w1[j][c];
+                        sh->band[e][9 + c][i] = w2[j][c];
+                    }
+            }
+        }
+        cl.sync();
+#pragma unroll
+        for (int j = 0; j < M; ++j) {
+            const int m = m0 + j;
+            const bool before = m < lo, after = m >= hi && m < hi + halo && rank < C - 1;
+            if (before || after) {
+                const Shared *from = cl.map_shared_rank(sh, before ? rank - 1 : rank + 1);
+                const R(*b)[kMaxHalo] = reinterpret_cast<const R(*)[kMaxHalo]>(from->band[before ? 1 : 0]);
+                const int i = before ? m - (lo - halo) : m - hi;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    y1[j][c] = b[c][i];
+                    y2[j][c] = b[3 + c][i];
+                    w1[j][c] = b[6 + c][i];
+                    w2[j][c] = b[9 + c][i];
+                }
+            }
+        }
+        cl.sync();             // the bands may be written again
+    }
 
     template <class LoadK, class Store>
-    __device__ __forceinline__ void project(const RegShot &sh, const MomentumTables &mom,
+    __device__ __forceinline__ void project(const RegShot &sh_, const MomentumTables &mom,
                                             LoadK loadk, Store store)
     {
-        project_registers<R, M>(sh, mom, first_sample(), mine, to_right, to_left, first, last,
-                                [] { sync(); }, loadk, store);
-        sync();                // the slots are free again (and no CTA leaves early)
+        const int m0 = first_sample();
+        project_registers<R, M>(
+            sh_, mom, m0, mine, to_right, to_left, first, last,
+            [] { if (CL == kMeet) cluster_sync(); else cta_sync(); },
+            [&](int it, R (*y1)[3], R (*y2)[3], R (*w1)[3], R (*w2)[3]) {
+                refresh(it, m0, y1, y2, w1, w2);
+            },
+            loadk, [&](int m, const R *s) { if (owns(m)) store(m, s); });
+        cluster_sync();        // the slots are free again (and no CTA leaves early)
     }
 };
 
 // One shot per cluster (CL) or CTA, grid-stride over shots; thread t of CTA
 // rank r owns samples (r * blockDim + t) * M + [0, M).
-template <class R, int M, typename KT, bool CL>
-__global__ void __launch_bounds__(reg_max_threads(M)) project_reg_kernel(const ProjArgs p)
+template <class R, int M, typename KT, int CL>
+__global__ void __launch_bounds__(reg_max_threads(M)) project_reg_kernel(const ProjArgs p,
+                                                                         const RegShape shape)
 {
-    __shared__ EdgeSlot<R> slots[reg_max_threads(M) / 32];
-    RegEdges<R, M, CL> edges(slots);
+    __shared__ typename RegEdges<R, M, CL>::Shared shared;
+    RegEdges<R, M, CL> edges(&shared, shape);
     RegShot sh;
     sh.Ns = p.Ns; sh.n_iter = p.n_iter; sh.pin_index = p.pin_index;
     sh.alpha = p.alpha; sh.beta = p.beta; sh.box = p.box;
@@ -159,14 +244,15 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_reg_kernel(const P
 // gradient is formed from the trajectory's slots and repulsion totals in the
 // order of the engine's projection items.  A trajectory whose pair items did
 // not all finish (a bounded wait ran out) is left as it is.
-template <int M, bool CL>
+template <int M, int CL>
 __global__ void __launch_bounds__(reg_max_threads(M)) project_batch_kernel(const EngineArgs e,
                                                                            int B, int64_t shots,
                                                                            int Ns,
-                                                                           MomentumTables mom)
+                                                                           MomentumTables mom,
+                                                                           const RegShape shape)
 {
-    __shared__ EdgeSlot<Df> slots[reg_max_threads(M) / 32];
-    RegEdges<Df, M, CL> edges(slots);
+    __shared__ typename RegEdges<Df, M, CL>::Shared shared;
+    RegEdges<Df, M, CL> edges(&shared, shape);
     for (int64_t shot = blockIdx.x / edges.C; shot < shots; shot += gridDim.x / edges.C) {
         int lo = 0, hi = B - 1;                   // the largest t with off_t <= shot * Ns
         while (lo < hi) {
@@ -221,7 +307,7 @@ __global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
         record_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * (int64_t)p.Ns, sp);
 }
 
-template <bool CL> void *reg_fn(int dtype, int M)
+template <int CL> void *reg_fn(int dtype, int M)
 {
     if (dtype == 0)
         return M == 1 ? reinterpret_cast<void *>(project_reg_kernel<Df, 1, float, CL>)
@@ -246,6 +332,40 @@ bool project_reg_applies(int dtype, int Ns, double alpha, double beta, double bo
     return true;
 }
 
+namespace {
+
+// Shape of one shot over C CTAs with halos (at least 8 samples, 3 iterations
+// between copies); false where it does not fit.
+bool reg_halo_shape(int Ns, int M, int C, RegShape &s)
+{
+    const int sides = C == 2 ? 1 : 2;            // of two CTAs each has one neighbour
+    s.per_thread = M;
+    s.ctas = C;
+    s.own = (Ns + C - 1) / C;
+    s.threads = ((s.own + 8 * sides + M - 1) / M + 31) / 32 * 32;
+    s.halo = (s.threads * M - s.own) / sides;
+    s.halo = s.halo < kMaxHalo ? s.halo : kMaxHalo;
+    s.halo = s.halo < s.own ? s.halo : s.own;
+    // every CTA owns samples, and the last one holds what its neighbour needs
+    return s.threads <= reg_max_threads(M) && s.halo >= 8 && Ns - (C - 1) * s.own >= s.halo;
+}
+
+// Time of 100 iterations (us) where every CTA has an SM to itself: a chain's
+// latency, or the issue of the SM's warps (FP64: of its FP64 pipe); ~0.5 us a
+// cluster barrier, of which a shape with halos has two a copy.  Fitted to
+// shots of 64 .. 2560 samples.
+double reg_time(bool fp64, const RegShape &s)
+{
+    const int w = s.threads / 32;
+    const bool one = s.per_thread == 1;
+    const double chain = fp64 ? (one ? 310.0 : 550.0) : one ? 88.0 : 108.0;
+    const double warp = fp64 ? (one ? 72.0 : 122.0) : one ? 14.0 : 19.0;
+    const double barriers = s.halo ? 300.0 / ((s.halo - 2) / 2) : s.ctas > 1 ? 90.0 : 0.0;
+    return (w * warp > chain ? w * warp : chain) + barriers;
+}
+
+} // namespace
+
 // Shape rule.  Two floats (FP32 samples): issue-bound, so M = 2 (the fewest
 // instructions a sample), and CTAs of at most 256 threads -- two on an SM
 // cover each other's barriers: 4096 shots of 2560 samples take 24.5 ms as 5
@@ -256,7 +376,10 @@ bool project_reg_applies(int dtype, int Ns, double alpha, double beta, double bo
 // where the shots do not fill the GPU (37 x 129: 379 against 531 us; 300 x
 // 700: 2.80 against 2.53 ms).  One CTA up to 1024 samples (a cluster barrier
 // costs ~0.4 us: 300 x 700 as 2 CTAs takes 2.79 ms), else at most 256 threads.
-RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms)
+// Few shots (`halos`; every CTA with an SM to itself): more, smaller CTAs a
+// shot with halos, as the times above say.  FP64 8 x 1000 1891 -> 410 us, 20 x
+// 500 985 -> 338, 37 x 129 381 -> 315; FP32 1 x 512 164 -> 120, 8 x 2560 238 -> 184.
+RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms, bool halos)
 {
     RegShape s;
     const bool fp64 = dtype != 0;
@@ -266,6 +389,18 @@ RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms)
     if (s.ctas > kRegMaxCtas) s.ctas = kRegMaxCtas;
     const int per = s.ctas * s.per_thread;
     s.threads = ((Ns + per - 1) / per + 31) / 32 * 32;
+    if (!halos) return s;
+    double best = 0.95 * reg_time(fp64, s);
+    for (int M = 1; M <= 2; ++M)
+        for (int C = 2; C <= kRegMaxCtas && Nc * C <= sms; ++C) {
+            RegShape h;
+            if (!reg_halo_shape(Ns, M, C, h)) continue;
+            const double t = reg_time(fp64, h);
+            if (t < best) {
+                best = t;
+                s = h;
+            }
+        }
     return s;
 }
 
@@ -292,21 +427,22 @@ cudaError_t launch_reg(void *fn, const RegShape &s, int64_t shots, void **args, 
 cudaError_t launch_project_batch(const EngineArgs &e, int32_t B, int64_t shots, int Ns,
                                  const MomentumTables &mom, const RegShape &s, cudaStream_t st)
 {
-    void *fn = s.ctas > 1 ? (s.per_thread == 1 ? reinterpret_cast<void *>(project_batch_kernel<1, true>)
-                                               : reinterpret_cast<void *>(project_batch_kernel<2, true>))
-                          : (s.per_thread == 1 ? reinterpret_cast<void *>(project_batch_kernel<1, false>)
-                                               : reinterpret_cast<void *>(project_batch_kernel<2, false>));
+    void *fn = s.ctas > 1 ? (s.per_thread == 1 ? reinterpret_cast<void *>(project_batch_kernel<1, kMeet>)
+                                               : reinterpret_cast<void *>(project_batch_kernel<2, kMeet>))
+                          : (s.per_thread == 1 ? reinterpret_cast<void *>(project_batch_kernel<1, kAlone>)
+                                               : reinterpret_cast<void *>(project_batch_kernel<2, kAlone>));
     int b = B;
     MomentumTables m = mom;
-    void *args[] = {const_cast<EngineArgs *>(&e), &b, &shots, &Ns, &m};
+    void *args[] = {const_cast<EngineArgs *>(&e), &b, &shots, &Ns, &m, const_cast<RegShape *>(&s)};
     return launch_reg(fn, s, shots, args, st);
 }
 
 cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, int sms,
                                cudaStream_t st)
 {
-    void *fn = s.ctas > 1 ? reg_fn<true>(dtype, s.per_thread) : reg_fn<false>(dtype, s.per_thread);
-    void *args[] = {const_cast<ProjArgs *>(&p)};
+    void *fn = s.halo ? reg_fn<kHalo>(dtype, s.per_thread)
+               : s.ctas > 1 ? reg_fn<kMeet>(dtype, s.per_thread) : reg_fn<kAlone>(dtype, s.per_thread);
+    void *args[] = {const_cast<ProjArgs *>(&p), const_cast<RegShape *>(&s)};
     cudaError_t e = launch_reg(fn, s, p.Nc, args, st);
     if (e != cudaSuccess || !p.viol) return e;
     const unsigned g = (unsigned)(p.Nc < sms * 8 ? p.Nc : sms * 8);

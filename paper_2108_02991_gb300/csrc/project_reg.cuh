@@ -259,12 +259,14 @@ struct RegShot {
 // neighbour's a, its left neighbour's b; null at the ends of the shot),
 // possibly in another CTA of the cluster.  first / last: no warp on that
 // side; the slots nobody writes are zero.  loadk(m, kv) gives the FP64 input; store(m, s) takes the result.
-template <class R, int M, class Sync, class LoadK, class Store>
+// refresh(it, y1, y2, w1, w2) may replace the state after iteration it (-1:
+// once the input is loaded).
+template <class R, int M, class Sync, class Refresh, class LoadK, class Store>
 __device__ __forceinline__ void project_registers(const RegShot &p, const MomentumTables &mom, int m0,
                                                   EdgeSlot<R> *mine,
                                                   EdgeSlot<R> *to_right, EdgeSlot<R> *to_left,
-                                                  bool first, bool last, Sync sync, LoadK loadk,
-                                                  Store store)
+                                                  bool first, bool last, Sync sync, Refresh refresh,
+                                                  LoadK loadk, Store store)
 {
     constexpr bool kTwoFloat = std::is_same<R, Df>::value;
     const int lane = threadIdx.x & 31;
@@ -290,6 +292,7 @@ __device__ __forceinline__ void project_registers(const RegShot &p, const Moment
             y1[j][c] = y2[j][c] = w1[j][c] = w2[j][c] = r_zero<R>();
         }
     }
+    refresh(-1, y1, y2, w1, w2);
     const bool pinned = p.pin_index >= m0 && p.pin_index < m0 + M;
     for (int it = 0;; ++it) {
         // s from (Y1, Y2): dp[j] = D^T Y of the thread's samples
@@ -397,6 +400,7 @@ __device__ __forceinline__ void project_registers(const RegShot &p, const Moment
                     y2[j][c] = w2[j][c];
                 }
         }
+        if (!final) refresh(it, y1, y2, w1, w2);
     }
 #pragma unroll
     for (int j = 0; j < M; ++j)

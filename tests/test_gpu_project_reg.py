@@ -84,6 +84,17 @@ def test_more_iterations_than_the_momentum_table(sp, ctx):
     check(sp, ctx, shots(5, 150, 7, 5e-3), 5, 150, np.float32, 2e-3, 1e-5, 4200)
 
 
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("Nc,Ns,n_iter", [(1, 96, 1), (1, 97, 2), (1, 300, 37), (2, 512, 100), (5, 777, 64),
+                                          (7, 1000, 100), (18, 500, 60), (37, 129, 100), (76, 130, 33),
+                                          (3, 2560, 60), (1, 4095, 50), (2, 8190, 30)])
+def test_few_shots_over_many_ctas(sp, ctx, Nc, Ns, n_iter, dt):
+    """Shots split over CTAs that also compute a halo of their neighbours:
+    owners' bands, copies every few iterations, none at all, pins in a halo."""
+    a, b = 1.0 / (2 * Ns), 1.0 / (8 * Ns * Ns)
+    check(sp, ctx, shots(Nc, Ns, Nc + Ns, 4.0 * a), Nc, Ns, dt, a, b, n_iter, pin_index=Ns // 2)
+
+
 def test_more_shots_than_a_grid_holds_at_once(sp, ctx):
     check(sp, ctx, shots(1500, 33, 3, 0.02), 1500, 33, np.float32, 1 / 66, 1 / 8712, 30)
 

@@ -95,9 +95,10 @@ constexpr int kMaxHalo = 32;
 // The slots and neighbours of the calling warp; zeroed, and every CTA of the
 // cluster running, on return.
 template <class R, int M, int CL> struct RegEdges {
+    typedef typename VecOf<R>::type V;
     struct Shared {
         EdgeSlot<R> slots[reg_max_threads(M) / 32];
-        R band[CL == kHalo ? 2 : 1][CL == kHalo ? 12 : 1][CL == kHalo ? kMaxHalo : 1];
+        V band[CL == kHalo ? 2 : 1][CL == kHalo ? 4 : 1][CL == kHalo ? kMaxHalo : 1];
     };
     Shared *sh;
     EdgeSlot<R> *mine, *to_right = nullptr, *to_left = nullptr;
@@ -147,8 +148,7 @@ template <class R, int M, int CL> struct RegEdges {
     // Every (halo - 2) / 2 iterations: the owners' state of the halos' samples.
     // (Before the first one, too: no CTA may store its result over samples that a
     // neighbour has still to load for its halo.)
-    __device__ __forceinline__ void refresh(int it, int m0, R (*y1)[3], R (*y2)[3], R (*w1)[3],
-                                            R (*w2)[3])
+    __device__ __forceinline__ void refresh(int it, int m0, V *y1, V *y2, V *w1, V *w2)
     {
         if (CL != kHalo || (it + 1) % ((halo - 2) / 2) != 0) return;
         namespace cg = cooperative_groups;
@@ -161,14 +161,12 @@ template <class R, int M, int CL> struct RegEdges {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int i = e == 0 ? m - lo : m - (hi - halo);
-                if (m >= lo && m < hi && i >= 0 && i < halo)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        sh->band[e][c][i] = y1[j][c];
-                        sh->band[e][3 + c][i] = y2[j][c];
-                        sh->band[e][6 + c][i] = w1[j][c];
-                        sh->band[e][9 + c][i] = w2[j][c];
-                    }
+                if (m >= lo && m < hi && i >= 0 && i < halo) {
+                    sh->band[e][0][i] = y1[j];
+                    sh->band[e][1][i] = y2[j];
+                    sh->band[e][2][i] = w1[j];
+                    sh->band[e][3][i] = w2[j];
+                }
             }
         }
         cl.sync();
@@ -178,15 +176,12 @@ template <class R, int M, int CL> struct RegEdges {
             const bool before = m < lo, after = m >= hi && m < hi + halo && rank < C - 1;
             if (before || after) {
                 const Shared *from = cl.map_shared_rank(sh, before ? rank - 1 : rank + 1);
-                const R(*b)[kMaxHalo] = reinterpret_cast<const R(*)[kMaxHalo]>(from->band[before ? 1 : 0]);
+                const V(*b)[kMaxHalo] = reinterpret_cast<const V(*)[kMaxHalo]>(from->band[before ? 1 : 0]);
                 const int i = before ? m - (lo - halo) : m - hi;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    y1[j][c] = b[c][i];
-                    y2[j][c] = b[3 + c][i];
-                    w1[j][c] = b[6 + c][i];
-                    w2[j][c] = b[9 + c][i];
-                }
+                y1[j] = b[0][i];
+                y2[j] = b[1][i];
+                w1[j] = b[2][i];
+                w2[j] = b[3][i];
             }
         }
         cl.sync();             // the bands may be written again
@@ -200,10 +195,10 @@ template <class R, int M, int CL> struct RegEdges {
         project_registers<R, M>(
             sh_, mom, m0, mine, to_right, to_left, first, last,
             [] { if (CL == kMeet) cluster_sync(); else cta_sync(); },
-            [&](int it, R (*y1)[3], R (*y2)[3], R (*w1)[3], R (*w2)[3]) {
+            [&](int it, V *y1, V *y2, V *w1, V *w2) {
                 refresh(it, m0, y1, y2, w1, w2);
             },
-            loadk, [&](int m, const R *s) { if (owns(m)) store(m, s); });
+            loadk, [&](int m, const V &s) { if (owns(m)) store(m, s); });
         cluster_sync();        // the slots are free again (and no CTA leaves early)
     }
 };
@@ -233,9 +228,11 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_reg_kernel(const P
                     if (G) kv[c] -= eta * G[3 * (off + m) + c];
                 }
             },
-            [&](int m, const R *s) {
+            [&](int m, const typename VecOf<R>::type &s) {
+                KT o[3];
+                v_values(s, o);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) K[3 * (off + m) + c] = (KT)r_value(s[c]);
+                for (int c = 0; c < 3; ++c) K[3 * (off + m) + c] = o[c];
             });
     }
 }
@@ -287,9 +284,11 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_batch_kernel(const
                 }
                 for (int c = 0; c < 3; ++c) kv[c] = (double)K[3 * m + c] - eta * (g[c] - r[c] * invN);
             },
-            [&](int m, const Df *s) {
+            [&](int m, const VecDf &s) {
+                float o[3];
+                v_values(s, o);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) K[3 * m + c] = r_value(s[c]);
+                for (int c = 0; c < 3; ++c) K[3 * m + c] = o[c];
             });
     }
 }
@@ -368,9 +367,10 @@ double reg_time(bool fp64, const RegShape &s)
 
 // Shape rule.  Two floats (FP32 samples): issue-bound, so M = 2 (the fewest
 // instructions a sample), and CTAs of at most 256 threads -- two on an SM
-// cover each other's barriers: 4096 shots of 2560 samples take 24.5 ms as 5
-// CTAs of 256 threads, 30.1 ms as 3 of 448.  Shots of up to 128 samples are
-// bound by the latency of one warp's chain: M = 1 (32 x 64: 86 against 107 us).
+// cover each other's barriers: 4096 shots of 2560 samples take 21.9 ms as 5
+// CTAs of 256 threads (before x and y were paired: 24.5 ms, and 30.1 ms as 3 of
+// 448).  Shots of up to 128 samples are bound by the latency of one warp's
+// chain: M = 1 (32 x 64: 86 against 107 us, then too).
 // FP64: bound by the FP64 pipe, which every warp of an SM shares.  M = 1 costs
 // ~10 % more operations but pads less and has the shorter chain; it is taken
 // where the shots do not fill the GPU (37 x 129: 379 against 531 us; 300 x

@@ -73,7 +73,8 @@ def parse_args(argv=None):
                     help="batched step: the symmetric repulsion in its own kernel ahead of the "
                          "engine instead of as items of the engine's work list (one launch)")
     ap.add_argument("--projection", choices=("fp64", "mixed"), default="fp64",
-                    help="projection arithmetic: FP64 duals (default) or the opt-in mixed form")
+                    help="projection arithmetic: the default (FP64, two-float sums for FP32 samples) or "
+                         "mixed (an FP32 iteration is allowed)")
     ap.add_argument("--shot-stride", type=int, default=1,
                     help="keep every S-th shot of the workload (same density): a smaller launch "
                          "of the same kernels, e.g. for a profiler capture")
@@ -671,7 +672,7 @@ def run_ours(args):
     if rank == 0:
         p0 = w.probs[0]
         proj_form = ("mixed FP32/FP64 projection" if args.projection == "mixed"
-                     else "FP64 projection (duals, primal, step)")
+                     else "FP64 projection step, duals and primal in two-float sums (48 bits)")
         acc_form = {"kahan": "compensated-f32 per-target sums",
                     "fp64": "f64 per-target sums of f32 row sums",
                     "fp64pair": "every attraction pair term added in f64"}[args.acc]

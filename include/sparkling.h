@@ -127,7 +127,7 @@ typedef struct sparkling_proj {
 #define SPARKLING_KERNEL_REPULSION 2
 #define SPARKLING_KERNEL_COMBINE 3
 #define SPARKLING_KERNEL_PROJECT 4
-#define SPARKLING_KERNEL_ENGINE 5   /* a whole batched step (packs + persistent engine) */
+#define SPARKLING_KERNEL_ENGINE 5   /* a whole batched step (packs + persistent engine + projection) */
 #define SPARKLING_KERNEL_DRIVER 6   /* up-sampling and step-size reductions of the driver */
 #define SPARKLING_KERNEL_STEP 7     /* the whole device work of one sparkling_step call */
 #define SPARKLING_KERNEL_COUNT 8
@@ -139,7 +139,7 @@ typedef struct sparkling_proj {
 /* How sparkling_step runs its device work (sparkling_set_step_path). */
 #define SPARKLING_STEP_AUTO 0      /* the persistent engine from 2^22 samples on, else the kernels (default) */
 #define SPARKLING_STEP_KERNELS 1   /* attraction, repulsion, combine and projection kernels in turn */
-#define SPARKLING_STEP_ENGINE 2    /* the one-launch persistent engine wherever it applies */
+#define SPARKLING_STEP_ENGINE 2    /* the persistent engine wherever it applies */
 
 /* How the attraction term is evaluated (sparkling_set_attraction). */
 #define SPARKLING_ATTRACTION_DIRECT 0   /* direct sum over the grid: O(N P) */
@@ -254,11 +254,12 @@ SPARKLING_API int sparkling_project(sparkling_ctx *ctx, void *K, int K_dtype, in
  * (so eta = 1/N is a unit step on dF/dK).  The gradient is kept in FP64 in
  * the workspace; the step and the projection run in FP64 (unless the
  * context chose SPARKLING_PROJECTION_MIXED) and the result is rounded to
- * K_dtype.  With timing on, the device work of the call is also timed as one
+ * K_dtype (two-float sums for FP32 K: sparkling_set_projection).  With timing on, the device work of the call is also timed as one
  * SPARKLING_KERNEL_STEP scope.  The device work runs either as the separate
- * kernels or as one launch of the persistent engine (sparkling_step_batched
- * with B = 1: the same arithmetic, attraction and symmetric repulsion items
- * sharing the SMs), as sparkling_set_step_path chooses; the engine applies
+ * kernels or on the persistent engine (sparkling_step_batched with B = 1: the
+ * same arithmetic, attraction and symmetric repulsion items of one launch
+ * sharing the SMs, FP32 samples projected by a second launch), as
+ * sparkling_set_step_path chooses; the engine applies
  * with direct sums, ACC_KAHAN32 or ACC_FP64 and a fixed n_iter.
  * Asynchronous on the kernels path unless converged mode is requested; the
  * engine path first waits for the stream's earlier work. */
@@ -267,8 +268,8 @@ SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64
                                  const sparkling_proj *proj, void *stream);
 
 /* One projected-gradient step K_b <- Pi(K_b - eta_b G(K_b)) for B
- * independent trajectories of uneven size in one persistent launch (plus
- * the packing of samples and densities): a work list of attraction items (a
+ * independent trajectories of uneven size on the persistent engine (after
+ * the packing of samples and densities): one launch runs a work list of attraction items (a
  * tile of 1024 targets against a run of grid rows) and symmetric repulsion
  * items (a tile of targets against a run of source tiles, each unordered
  * pair once, exact fixed-point totals per sample).  FP32 trajectories are
@@ -420,7 +421,7 @@ SPARKLING_API int sparkling_set_regularisation(sparkling_ctx *ctx, double eps);
 SPARKLING_API int sparkling_set_projection(sparkling_ctx *ctx, int mode);
 
 /* Device path of the context's sparkling_step and sparkling_step_host calls
- * (SPARKLING_STEP_*).  AUTO (default) takes the one-launch persistent engine
+ * (SPARKLING_STEP_*).  AUTO (default) takes the persistent engine
  * for steps of 2^22 samples or more (on the 1e7-sample workload it is ~8 %
  * faster than the kernels in turn, since SFU-bound attraction items and
  * FP32-bound repulsion items share each SM) and the kernels below that;
@@ -477,7 +478,7 @@ SPARKLING_API int sparkling_set_attraction(sparkling_ctx *ctx, int mode);
  *     fast multipole method (Sec. II-C.2), a particle-particle particle-mesh
  *     split of the kernel d/|d|_eps = d/r erfc(r/sigma) + d/r erf(r/sigma):
  *     the first part is summed directly over the pairs closer than
- *     rc = rc_sigmas * sigma (a cell list), the second on the mesh (cubic
+ *     rc = rc_sigmas * sigma (clusters of sorted samples), the second on the mesh (cubic
  *     B-spline charges, FP32 FFT convolution with a deconvolved, tapered
  *     kernel, interpolation back); the energy the same way with the matching
  *     potential.  Approximate: its error against the direct sum is measured
@@ -491,8 +492,7 @@ SPARKLING_API int sparkling_set_attraction(sparkling_ctx *ctx, int mode);
  *     outside any stream capture they can be captured into a CUDA graph.  A
  *     captured call that would have to size buffers returns
  *     SPARKLING_E_INVAL; a graph captured before a call with a larger sample
- *     count (which resizes them) must be
- *     captured again.
+ *     count (which resizes them) must be captured again.
  * Returns SPARKLING_E_INVAL for a bad mode or mesh. */
 SPARKLING_API int sparkling_set_repulsion(sparkling_ctx *ctx, int mode, const sparkling_mesh *mesh);
 

@@ -1477,8 +1477,8 @@ SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64
         return fail(ctx, SPARKLING_E_INVAL, "K and grid->rho must be device memory");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t N = Nc * Ns;
-    // The persistent engine takes the whole step in one launch (B = 1) where
-    // it applies: direct sums, a per-target fold it has, fixed iterations.
+    // The persistent engine takes the whole step (B = 1) where it applies:
+    // direct sums, a per-target fold it has, fixed iterations.
     const bool engine_applies = ctx->attr_mode == SPARKLING_ATTRACTION_DIRECT &&
                                 ctx->rep_mode == SPARKLING_REPULSION_DIRECT &&
                                 (acc == SPARKLING_ACC_KAHAN32 || acc == SPARKLING_ACC_FP64) &&

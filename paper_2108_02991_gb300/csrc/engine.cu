@@ -4,7 +4,10 @@
 //
 // The host builds a work list (api.cu): for every trajectory and every tile
 // of 1024 targets, attraction items (a run of grid rows), then one
-// projection item per shot.  The repulsion of every trajectory is summed
+// projection item per shot -- unless the samples are FP32 and in the range of
+// the register form, whose projections are a second launch (project.cu): with
+// that form inside this kernel the pair loops got other registers and the
+// pair items of 16 trajectories took 250 ms instead of 224.  The repulsion of every trajectory is summed
 // with each unordered pair once, into exact fixed-point totals per sample
 // (EngineArgs::racc): in the one-launch shape by symmetric repulsion items
 // of the same work list (a target tile against a run of source tiles),

@@ -297,8 +297,9 @@ cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, 
 // Persistent engine (engine.cu): one launch runs a work list of pair items
 // (attraction or repulsion of one target tile against a run of grid rows or
 // source blocks, or symmetric repulsion of one target tile against a run of
-// source tiles) for any number of trajectories, followed by per-shot
-// projection items that wait until their trajectory's pair items are done.
+// source tiles) for any number of trajectories, followed (where the projection
+// is not a launch of its own, launch_project_batch) by per-shot projection
+// items that wait until their trajectory's pair items are done.
 struct EngineTraj {
     int64_t off;             // first sample of the trajectory in K / pos
     int64_t N;               // samples

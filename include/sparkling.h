@@ -222,12 +222,33 @@ SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, i
                                             const double *g_dev, double scale, void *dK,
                                             int dK_dtype, void *stream);
 
-/* sparkling_energy and its gradient together, for automatic differentiation:
- * where one pass over the pairs of the attraction gives both (direct sums,
- * ACC_KAHAN32 or ACC_FP64), also writes dK = dF/dK = (A - R) / N, [N][3] of
- * double on the device, and sets *wrote = 1; otherwise only the energy is
- * computed and *wrote = 0 (use sparkling_energy_backward).  Blocks on
- * `stream`. */
+/* For automatic differentiation: sparkling_energy that keeps the attraction's
+ * sums for a backward that may follow.  Where sparkling_keeps_attraction(ctx,
+ * acc) is 1 (direct sums, ACC_KAHAN32 or ACC_FP64) one pass over the
+ * attraction's pairs gives the energy and A, [N][3] of double on the device,
+ * and *A_eps becomes the regularisation that A holds for; elsewhere, or with A
+ * or A_eps NULL, the call is sparkling_energy and *A_eps becomes -1.  The pass takes 4 to 9 % longer
+ * than the energy's own, the backward is left with the repulsion. */
+SPARKLING_API int sparkling_keeps_attraction(const sparkling_ctx *ctx, int acc);
+SPARKLING_API int sparkling_energy_keep(sparkling_ctx *ctx, const void *K, int K_dtype, int64_t N,
+                                        const sparkling_grid *grid, int acc, double *F_host,
+                                        double *Fa_host, double *Fr_host, double *A, double *A_eps,
+                                        void *stream);
+
+/* sparkling_energy_backward with the attraction's sums of the same K, grid and
+ * acc at hand (A and *A_eps of sparkling_energy_keep).  The context's settings
+ * at this call count: where they are not those that A was formed with, or A is
+ * NULL, the attraction is summed again. */
+SPARKLING_API int sparkling_energy_backward_kept(sparkling_ctx *ctx, const void *K, int K_dtype,
+                                                 int64_t N, const sparkling_grid *grid, int acc,
+                                                 const double *A, double A_eps, const double *g_dev,
+                                                 double scale, void *dK, int dK_dtype, void *stream);
+
+/* sparkling_energy and its gradient together: where one pass over the pairs of
+ * the attraction gives both (sparkling_keeps_attraction), also writes dK =
+ * dF/dK = (A - R) / N, [N][3] of double on the device, and sets *wrote = 1;
+ * otherwise only the energy is computed and *wrote = 0 (use
+ * sparkling_energy_backward).  Blocks on `stream`. */
 SPARKLING_API int sparkling_energy_and_grad(sparkling_ctx *ctx, const void *K, int K_dtype,
                                             int64_t N, const sparkling_grid *grid, int acc,
                                             double *F_host, double *Fa_host, double *Fr_host,

@@ -30,7 +30,8 @@ REPULSION_DIRECT, REPULSION_MESH = 0, 1
 # Every entry point declared in include/sparkling.h.
 ABI_SYMBOLS = (
     "sparkling_create", "sparkling_destroy", "sparkling_last_error", "sparkling_grad",
-    "sparkling_energy", "sparkling_energy_backward", "sparkling_energy_and_grad", "sparkling_project", "sparkling_step",
+    "sparkling_energy", "sparkling_energy_backward", "sparkling_keeps_attraction", "sparkling_energy_keep",
+    "sparkling_energy_backward_kept", "sparkling_energy_and_grad", "sparkling_project", "sparkling_step",
     "sparkling_step_host", "sparkling_status", "sparkling_set_timing", "sparkling_kernel_times",
     "sparkling_launch_count", "sparkling_version", "sparkling_grad_noalloc",
     "sparkling_step_batched", "sparkling_set_autotune", "sparkling_tuning_report",
@@ -113,6 +114,10 @@ def lib() -> ctypes.CDLL:
             "sparkling_grad": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, i, p, p, p], i),
             "sparkling_energy": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, p, p, p], i),
             "sparkling_energy_backward": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, d, p, i, p], i),
+            "sparkling_keeps_attraction": ([p, i], i),
+            "sparkling_energy_keep": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, p, p, p, p, p], i),
+            "sparkling_energy_backward_kept": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, d, p, d, p, i,
+                                                p], i),
             "sparkling_energy_and_grad": ([p, p, i, i64, ctypes.POINTER(Grid), i, p, p, p, p, p, p], i),
             "sparkling_project": ([p, p, i, i64, i64, ctypes.POINTER(Proj), p, p], i),
             "sparkling_step": ([p, p, i, i64, i64, ctypes.POINTER(Grid), i, d, ctypes.POINTER(Proj), p], i),
@@ -306,6 +311,44 @@ def sparkling_energy_backward(ctx: Context, K, grid: Grid, g=None, scale: float 
     _check(ctx, lib().sparkling_energy_backward(
         ctx.handle, _dev_ptr(K, "K"), _dtype_code(K), _rows(K), ctypes.byref(grid), acc,
         _dev_ptr(g, "g"), float(scale), _dev_ptr(dK, "dK"), _dtype_code(dK), _stream(stream)))
+    return dK
+
+
+def sparkling_keeps_attraction(ctx: Context, acc: int = ACC_KAHAN32) -> bool:
+    """Whether sparkling_energy_keep keeps the attraction's sums (direct sums)."""
+    return bool(lib().sparkling_keeps_attraction(ctx.handle, acc))
+
+
+def sparkling_energy_keep(ctx: Context, K, grid: Grid, acc: int = ACC_KAHAN32, stream=None):
+    """((F, F^a, F^r), A, eps): A the attraction's sums as float64 [N, 3] and the
+    regularisation they hold for, or None and -1; blocks on the stream."""
+    import torch
+    F, Fa, Fr, eps = ctypes.c_double(), ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
+    A = None
+    if sparkling_keeps_attraction(ctx, acc):
+        A = torch.empty(K.shape, dtype=torch.float64, device=K.device)
+    _check(ctx, lib().sparkling_energy_keep(
+        ctx.handle, _dev_ptr(K, "K"), _dtype_code(K), _rows(K), ctypes.byref(grid), acc,
+        ctypes.byref(F), ctypes.byref(Fa), ctypes.byref(Fr), _dev_ptr(A, "A"), ctypes.byref(eps),
+        _stream(stream)))
+    return (F.value, Fa.value, Fr.value), A, eps.value
+
+
+def sparkling_energy_backward_kept(ctx: Context, K, grid: Grid, A, eps: float, g=None,
+                                   scale: float = 1.0, acc: int = ACC_KAHAN32, dK=None, stream=None):
+    """sparkling_energy_backward with A and eps of sparkling_energy_keep."""
+    import torch
+    if dK is None:
+        dK = torch.empty_like(K)
+    for t, what in ((g, "g"), (A, "A")):
+        if t is not None and t.dtype != torch.float64:
+            raise TypeError(f"{what} must be a float64 tensor")
+    if A is not None and A.shape != K.shape:
+        raise ValueError("A must have K's shape")
+    _check(ctx, lib().sparkling_energy_backward_kept(
+        ctx.handle, _dev_ptr(K, "K"), _dtype_code(K), _rows(K), ctypes.byref(grid), acc,
+        _dev_ptr(A, "A"), float(eps), _dev_ptr(g, "g"), float(scale), _dev_ptr(dK, "dK"),
+        _dtype_code(dK), _stream(stream)))
     return dK
 
 

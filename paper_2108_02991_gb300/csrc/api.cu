@@ -461,10 +461,19 @@ int attr_choice_of(const sparkling_ctx *ctx, int acc, int gxp)
     return -1;
 }
 
+// What one evaluation of the pair sums gives.
+constexpr int kGradient = 0;
+constexpr int kEnergy = 1;
+constexpr int kBoth = 2;           // the attraction's energy and force from one pass
+constexpr int kEnergyKeep = 3;     // the same pass, of the repulsion the energy alone; the sums A are kept
+
+// The attraction kernel's MODE.
+int attraction_mode(int mode) { return mode == kEnergyKeep ? 2 : mode; }
+
 // Splits of the two pair kernels for the chosen tile shapes.
 void set_splits(sparkling_ctx *ctx, PairPlan &P, int acc, int mode, int va, int vr)
 {
-    const int e = mode;
+    const int e = attraction_mode(mode);
     const int64_t rows = (int64_t)P.ny * P.nz;
     const int64_t nblocks = (P.N + kSrcBlock - 1) / kSrcBlock;
     if (ctx->occ_attr[acc][e][va] < 1) va = kAttrDefault;   // a pinned shape that cannot be resident
@@ -472,10 +481,9 @@ void set_splits(sparkling_ctx *ctx, PairPlan &P, int acc, int mode, int va, int 
     P.vr = vr;
     P.spa = make_split(P.tiles, rows, (int64_t)ctx->sms * ctx->occ_attr[acc][e][va]);
     P.spr = make_split(P.tiles, nblocks,
-                       (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][mode == 1 ? 1 : 0][vr]);
+                       (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][mode == kEnergy || mode == kEnergyKeep ? 1 : 0][vr]);
 }
 
-// mode: the gradient (0), the energy (1), or both (2).
 int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, int mode,
                bool need_g64, PairPlan &P, Carve &cv)
 {
@@ -504,7 +512,7 @@ int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, 
     P.o_coords = cv.take(((size_t)P.gxp + P.ny + P.nz) * sizeof(float));
     P.o_parta = cv.take((size_t)part_units * kTile * sizeof(dacc4));
     P.o_partr = cv.take((size_t)part_units * kTile * sizeof(dacc4));
-    P.o_racc = cv.take((size_t)N * (mode == 2 ? 4 : 3) * sizeof(unsigned long long));
+    P.o_racc = cv.take((size_t)N * (mode == kBoth ? 4 : 3) * sizeof(unsigned long long));
     P.o_eblocks = cv.take((size_t)energy_blocks(N) * sizeof(double2));
     P.o_g64 = need_g64 ? cv.take((size_t)N * 3 * sizeof(double)) : 0;
     P.o_adir = ctx->attr_mode == SPARKLING_ATTRACTION_FIELD ? cv.take((size_t)N * sizeof(dacc4)) : 0;
@@ -747,11 +755,13 @@ int run_repulsion(sparkling_ctx *ctx, PairPlan &P, const float4 *pos, const RepA
 // pack -> (autotune) -> attraction -> repulsion -> combine (gradient) or
 // energy reduction.  In field mode the attraction is the interpolated node
 // field.
-// mode 0: gradient; 1: energy; 2: both, the attraction's from one pass (the
-// repulsion, at most as many pairs, takes one for each).
+// kBoth: the attraction's from one pass (the repulsion, at most as many pairs,
+// takes one for each).  kEnergyKeep: A takes the attraction's sums [N][3]
+// (double), which a gradient takes back as A_kept in place of the pass.
 int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_grid *g, int acc,
               int mode, PairPlan &P, void *G, int G_dtype, void *A, void *R, bool g64,
-              cudaStream_t st, double scale = 1.0, const double *scale_dev = nullptr)
+              cudaStream_t st, double scale = 1.0, const double *scale_dev = nullptr,
+              const double *A_kept = nullptr)
 {
     float4 *pos = at<float4>(ctx, P.o_pos);
     float *rho = at<float>(ctx, P.o_rho);
@@ -767,12 +777,15 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     const bool small = !mesh_mode && P.N <= kSmallRepulsion && !ctx->pin_sym;
     // fixed-point totals of the repulsion, cleared by the pack
     const bool totals = small || (!mesh_mode && ctx->rep_symmetric);
-    const int64_t n_totals = totals ? P.N * (mode == 2 ? 4 : mode == 1 ? 1 : 3) : 0;
+    const bool force = mode == kGradient || mode == kBoth, value = mode != kGradient;
+    const int64_t n_totals = totals ? P.N * ((force ? 3 : 0) + (value ? 1 : 0)) : 0;
     {
         LaunchScope ls(ctx, SPARKLING_KERNEL_PACK, st);
-        CK(launch_pack(K, K_dtype, P.N, pos, g->rho, P.nx, P.ny, P.nz, P.gxp, g->lo, g->hi, rho,
-                       coords, at<unsigned long long>(ctx, P.o_racc), n_totals, ctx->d_status,
-                       ctx->sms, st));
+        // with the attraction's sums at hand the density is not read
+        const bool d = A_kept == nullptr;
+        CK(launch_pack(K, K_dtype, P.N, pos, g->rho, d ? P.nx : 0, d ? P.ny : 0, d ? P.nz : 0,
+                       d ? P.gxp : 0, g->lo, g->hi, rho, coords,
+                       at<unsigned long long>(ctx, P.o_racc), n_totals, ctx->d_status, ctx->sms, st));
         ls.done();
     }
     AttrArgs aa{};
@@ -787,7 +800,7 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     ra.pos = pos; ra.N = P.N; ra.part = at<dacc4>(ctx, P.o_partr);
     ra.status = ctx->d_status;
     ra.eps2 = aa.eps2;
-    const bool need_a = !field_mode && attr_choice_of(ctx, acc, P.gxp) < 0,
+    const bool need_a = !field_mode && !A_kept && attr_choice_of(ctx, acc, P.gxp) < 0,
                need_r = !mesh_mode && !small && !ctx->rep_symmetric && ctx->rep_choice[rep_acc(acc)] < 0,
                need_s = !mesh_mode && !small && ctx->rep_symmetric && ctx->sym_choice < 0;
     if (ctx->autotune && (need_a || need_r || need_s)) {
@@ -807,13 +820,13 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     aa.sp = P.spa;
     ra.sp = P.spr;
     dacc4 *a_direct = field_mode ? at<dacc4>(ctx, P.o_adir) : nullptr;
-    {
+    if (!A_kept) {
         LaunchScope ls(ctx, SPARKLING_KERNEL_ATTRACTION, st);
         if (field_mode)
             CK(launch_interp(pos, P.N, ctx->field, P.nx, P.ny, P.nz, g->lo, g->hi, a_direct,
                              ctx->sms, st));
         else
-            CK(launch_attraction(aa, acc, mode, P.va, st));
+            CK(launch_attraction(aa, acc, attraction_mode(mode), P.va, st));
         ls.done();
     }
     CombineArgs cb{};
@@ -821,19 +834,26 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     cb.G = G; cb.A = A; cb.R = R;
     cb.G64 = g64 ? at<double>(ctx, P.o_g64) : nullptr;
     cb.a_direct = a_direct;
+    cb.a_kept = A_kept;
     cb.scale = scale;
     cb.scale_dev = scale_dev;
     cb.eps = ctx->eps;
     cb.energy_blocks = at<double2>(ctx, P.o_eblocks);
-    // the repulsion's force sums, then (mode 2) or instead (mode 1) its energy sums
-    for (int energy = mode == 1 ? 1 : 0; energy <= (mode == 0 ? 0 : 1); ++energy) {
+    if (mode == kEnergyKeep) {
+        cb.attraction_only = true;
+        LaunchScope ls(ctx, SPARKLING_KERNEL_COMBINE, st);
+        CK(launch_combine(cb, SPARKLING_F64, ctx->sms, st));
+        ls.done();
+    }
+    // the repulsion's force sums, its energy sums, or one after the other
+    for (int energy = force ? 0 : 1; energy <= (value ? 1 : 0); ++energy) {
         int s;
-        if (mode == 2 && energy)
+        if (mode == kBoth && energy)
             cb.spr = make_split(P.tiles, (P.N + kSrcBlock - 1) / kSrcBlock,
                                 (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][1][P.vr]);
         ra.sp = cb.spr;
         unsigned long long *racc = nullptr;
-        if (totals) racc = at<unsigned long long>(ctx, P.o_racc) + (mode == 2 && energy ? 3 * P.N : 0);
+        if (totals) racc = at<unsigned long long>(ctx, P.o_racc) + (mode == kBoth && energy ? 3 * P.N : 0);
         dacc4 *r_direct = nullptr;
         if ((s = run_repulsion(ctx, P, pos, ra, acc, energy != 0, small, racc, r_direct, st))) return s;
         cb.racc = racc;
@@ -1353,15 +1373,24 @@ SPARKLING_API int sparkling_grad(sparkling_ctx *ctx, const void *K, int K_dtype,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, 0, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, kGradient, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    return run_pairs(ctx, K, K_dtype, grid, acc, 0, P, G, G_dtype, A, R, false, st);
+    return run_pairs(ctx, K, K_dtype, grid, acc, kGradient, P, G, G_dtype, A, R, false, st);
 }
 
 SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, int K_dtype,
                                             int64_t N, const sparkling_grid *grid, int acc,
                                             const double *g_dev, double scale, void *dK,
                                             int dK_dtype, void *stream)
+{
+    return sparkling_energy_backward_kept(ctx, K, K_dtype, N, grid, acc, nullptr, -1.0, g_dev, scale,
+                                          dK, dK_dtype, stream);
+}
+
+SPARKLING_API int sparkling_energy_backward_kept(sparkling_ctx *ctx, const void *K, int K_dtype,
+                                                 int64_t N, const sparkling_grid *grid, int acc,
+                                                 const double *A, double A_eps, const double *g_dev,
+                                                 double scale, void *dK, int dK_dtype, void *stream)
 {
     int s;
     if ((s = common_checks(ctx, K, K_dtype, N, grid, acc))) return s;
@@ -1370,32 +1399,58 @@ SPARKLING_API int sparkling_energy_backward(sparkling_ctx *ctx, const void *K, i
     if (!std::isfinite(scale)) return fail(ctx, SPARKLING_E_INVAL, "scale must be finite");
     if ((s = lazy_init(ctx))) return s;
     if (!is_device_ptr(K) || !is_device_ptr(dK) || !is_device_ptr(grid->rho) ||
-        (g_dev && !is_device_ptr(g_dev)))
-        return fail(ctx, SPARKLING_E_INVAL, "K, dK, g_dev and grid->rho must be device memory");
+        (g_dev && !is_device_ptr(g_dev)) || (A && !is_device_ptr(A)))
+        return fail(ctx, SPARKLING_E_INVAL, "K, dK, g_dev, A and grid->rho must be device memory");
+    // the context's settings now are what counts, as without A
+    if (ctx->attr_mode != SPARKLING_ATTRACTION_DIRECT || acc == SPARKLING_ACC_FP64_PAIR ||
+        A_eps != ctx->eps)
+        A = nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, 0, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, kGradient, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    return run_pairs(ctx, K, K_dtype, grid, acc, 0, P, dK, dK_dtype, nullptr, nullptr, false, st,
-                     scale / (double)N, g_dev);
+    return run_pairs(ctx, K, K_dtype, grid, acc, kGradient, P, dK, dK_dtype, nullptr, nullptr, false, st,
+                     scale / (double)N, g_dev, A);
+}
+
+SPARKLING_API int sparkling_keeps_attraction(const sparkling_ctx *ctx, int acc)
+{
+    return ctx && ctx->attr_mode == SPARKLING_ATTRACTION_DIRECT &&
+                   ctx->rep_mode == SPARKLING_REPULSION_DIRECT &&
+                   (acc == SPARKLING_ACC_KAHAN32 || acc == SPARKLING_ACC_FP64)
+               ? 1
+               : 0;
 }
 
 SPARKLING_API int sparkling_energy(sparkling_ctx *ctx, const void *K, int K_dtype, int64_t N,
                                    const sparkling_grid *grid, int acc, double *F_host,
                                    double *Fa_host, double *Fr_host, void *stream)
 {
+    return sparkling_energy_keep(ctx, K, K_dtype, N, grid, acc, F_host, Fa_host, Fr_host, nullptr,
+                                 nullptr, stream);
+}
+
+SPARKLING_API int sparkling_energy_keep(sparkling_ctx *ctx, const void *K, int K_dtype, int64_t N,
+                                        const sparkling_grid *grid, int acc, double *F_host,
+                                        double *Fa_host, double *Fr_host, double *A, double *A_eps,
+                                        void *stream)
+{
     int s;
+    if (A_eps) *A_eps = -1.0;
     if ((s = common_checks(ctx, K, K_dtype, N, grid, acc))) return s;
     if ((s = lazy_init(ctx))) return s;
-    if (!is_device_ptr(K) || !is_device_ptr(grid->rho))
-        return fail(ctx, SPARKLING_E_INVAL, "K and grid->rho must be device memory");
+    if (!is_device_ptr(K) || !is_device_ptr(grid->rho) || (A && !is_device_ptr(A)))
+        return fail(ctx, SPARKLING_E_INVAL, "K, A and grid->rho must be device memory");
+    const bool keep = A && A_eps && sparkling_keeps_attraction(ctx, acc);
+    const int mode = keep ? kEnergyKeep : kEnergy;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, 1, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, mode, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 1, P, nullptr, 0, nullptr, nullptr, false, st)))
+    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, mode, P, nullptr, 0, keep ? A : nullptr, nullptr,
+                       false, st)))
         return s;
     double h[2];
     CK(cudaMemcpyAsync(h, ctx->d_small, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1403,6 +1458,7 @@ SPARKLING_API int sparkling_energy(sparkling_ctx *ctx, const void *K, int K_dtyp
     if (Fa_host) *Fa_host = h[0];
     if (Fr_host) *Fr_host = h[1];
     if (F_host) *F_host = h[0] - h[1];
+    if (keep) *A_eps = ctx->eps;
     return SPARKLING_OK;
 }
 
@@ -1416,8 +1472,7 @@ SPARKLING_API int sparkling_energy_and_grad(sparkling_ctx *ctx, const void *K, i
     if ((s = common_checks(ctx, K, K_dtype, N, grid, acc))) return s;
     if (!dK || !wrote) return fail(ctx, SPARKLING_E_INVAL, "dK and wrote are required");
     // one pass pays where it spares a second attraction sum of every pair
-    if (ctx->attr_mode != SPARKLING_ATTRACTION_DIRECT || ctx->rep_mode != SPARKLING_REPULSION_DIRECT ||
-        acc == SPARKLING_ACC_FP64_PAIR)
+    if (!sparkling_keeps_attraction(ctx, acc))
         return sparkling_energy(ctx, K, K_dtype, N, grid, acc, F_host, Fa_host, Fr_host, stream);
     if ((s = lazy_init(ctx))) return s;
     if (!is_device_ptr(K) || !is_device_ptr(dK) || !is_device_ptr(grid->rho))
@@ -1425,9 +1480,9 @@ SPARKLING_API int sparkling_energy_and_grad(sparkling_ctx *ctx, const void *K, i
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, 2, false, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, kBoth, false, P, cv))) return s;
     if ((s = ensure_ws(ctx, P.end))) return s;
-    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 2, P, dK, SPARKLING_F64, nullptr, nullptr, false, st,
+    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, kBoth, P, dK, SPARKLING_F64, nullptr, nullptr, false, st,
                        1.0 / (double)N)))
         return s;
     double h[2];
@@ -1495,13 +1550,13 @@ SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64
     }
     PairPlan P;
     Carve cv;
-    if ((s = plan_pairs(ctx, N, grid, acc, 0, true, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, kGradient, true, P, cv))) return s;
     ProjPlan L;
     if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     if ((s = ensure_ws(ctx, cv.off))) return s;
     // the whole device work of the step, timed as one scope when timing is on
     StepScope whole(ctx, st);
-    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 0, P, nullptr, K_dtype, nullptr, nullptr, true,
+    if ((s = run_pairs(ctx, K, K_dtype, grid, acc, kGradient, P, nullptr, K_dtype, nullptr, nullptr, true,
                        st)))
         return s;
     if ((s = run_project(ctx, K, K_dtype, Nc, Ns, proj, at<double>(ctx, P.o_g64), eta, L, false, st)))
@@ -1551,7 +1606,7 @@ int run_optimize(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t N
     PairPlan P;
     Carve cv;
     int s;
-    if ((s = plan_pairs(ctx, N, grid, acc, 0, true, P, cv))) return s;
+    if ((s = plan_pairs(ctx, N, grid, acc, kGradient, true, P, cv))) return s;
     ProjPlan L;
     if ((s = plan_project(ctx, K_dtype, Nc, Ns, proj, cv, L))) return s;
     const size_t o_kp = cv.take((size_t)n3 * sizeof(double));
@@ -1561,7 +1616,7 @@ int run_optimize(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t N
     const double *G64 = at<double>(ctx, P.o_g64);
     double step = sc->eta;
     for (int t = 0; t < sc->n_git; ++t) {
-        if ((s = run_pairs(ctx, K, K_dtype, grid, acc, 0, P, nullptr, K_dtype, nullptr, nullptr,
+        if ((s = run_pairs(ctx, K, K_dtype, grid, acc, kGradient, P, nullptr, K_dtype, nullptr, nullptr,
                            true, st)))
             return s;
         const bool bb = t >= sc->n_fixed && t > 0;

@@ -158,6 +158,8 @@ struct CombineArgs {
     double *G64;          // optional FP64 copy of G [N][3]
     const unsigned long long *racc;   // symmetric repulsion sums [N][NV] (replaces part_r)
     const dacc4 *a_direct;            // attraction per target [N] (replaces part_a), or null
+    const double *a_kept;             // the same as [N][3], or null
+    bool attraction_only;             // only A is asked for: the repulsion is not read
     const dacc4 *r_direct;            // repulsion sums per target [N] (replaces racc/part_r), or null
     double scale;         // G, A, R are multiplied by scale * (*scale_dev if set)
     const double *scale_dev;

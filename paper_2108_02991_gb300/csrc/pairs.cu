@@ -160,7 +160,9 @@ __device__ __forceinline__ void combine_sample(const CombineArgs &c, int64_t i, 
                                                double sc)
 {
     dacc4 r;
-    if (c.r_direct) {
+    if (c.attraction_only) {
+        r = make_dacc4(0.0, 0.0, 0.0, 0.0);
+    } else if (c.r_direct) {
         r = c.r_direct[i];
     } else if (c.racc) {
         r.x = (double)(long long)c.racc[3 * i] / kFixScale;
@@ -192,8 +194,12 @@ __global__ void combine_kernel(const CombineArgs c)
     const double invN = 1.0 / (double)c.N;
     const double sc = c.scale_dev ? c.scale * c.scale_dev[0] : c.scale;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < c.N;
-         i += (int64_t)gridDim.x * blockDim.x)
-        combine_sample<OT>(c, i, c.a_direct ? c.a_direct[i] : sum_slots(c.part_a, c.spa, i), invN, sc);
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const double *k = c.a_kept ? c.a_kept + 3 * i : nullptr;
+        combine_sample<OT>(c, i, k ? make_dacc4(k[0], k[1], k[2], 0.0)
+                                   : c.a_direct ? c.a_direct[i] : sum_slots(c.part_a, c.spa, i),
+                           invN, sc);
+    }
 }
 
 // Few samples: a tile's attraction is split over up to a whole wave of CTAs
@@ -430,7 +436,7 @@ constexpr int64_t kFewSamples = 1 << 16;
 // Threads a sample of the slot sums: 0 (one thread a sample, grid-stride), 8, 32.
 int slot_lanes(const CombineArgs &c)
 {
-    if (c.a_direct || c.spa.slots < kFewSlots || c.N > kFewSamples) return 0;
+    if (c.a_direct || c.a_kept || c.spa.slots < kFewSlots || c.N > kFewSamples) return 0;
     return c.spa.slots >= kManySlots ? 32 : 8;
 }
 int few_blocks(int64_t N, int lanes)

@@ -476,6 +476,10 @@ void set_splits(sparkling_ctx *ctx, PairPlan &P, int acc, int mode, int va, int 
     const int e = attraction_mode(mode);
     const int64_t rows = (int64_t)P.ny * P.nz;
     const int64_t nblocks = (P.N + kSrcBlock - 1) / kSrcBlock;
+    // The tuner times the force kernel.  With the energy beside it the shape of
+    // 512 threads is the fastest at every size (1024 samples on 32^3 to 196608
+    // on 75^3, 82750 on 96^3: 16.58 ms, 128 threads 17.59, 256 threads 17.29).
+    if (e == 2 && ctx->pin_attr < 0) va = kAttrBoth;
     if (ctx->occ_attr[acc][e][va] < 1) va = kAttrDefault;   // a pinned shape that cannot be resident
     P.va = va;
     P.vr = vr;
@@ -498,10 +502,10 @@ int plan_pairs(sparkling_ctx *ctx, int64_t N, const sparkling_grid *g, int acc, 
     // Partial buffers big enough for every tile shape and for the tuning
     // trials (which run on a prefix of the tiles with one wave of CTAs).
     int64_t max_ctas = 0;
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < 3; ++e) {
         for (int v = 0; v < kAttrVariants; ++v)
             max_ctas = std::max<int64_t>(max_ctas, (int64_t)ctx->sms * ctx->occ_attr[acc][e][v]);
-        for (int v = 0; v < kRepVariants; ++v)
+        for (int v = 0; v < kRepVariants && e < 2; ++v)
             max_ctas = std::max<int64_t>(max_ctas, (int64_t)ctx->sms * ctx->occ_rep[rep_acc(acc)][e][v]);
     }
     const int64_t part_units = std::max<int64_t>(P.tiles * ((max_ctas + P.tiles - 1) / P.tiles + 1),

@@ -174,6 +174,7 @@ struct CombineArgs {
 constexpr int kAttrVariants = 3;       // threads 128 / 256 / 512 (8 / 4 / 2 targets each)
 constexpr int kRepVariants = 5;        // (threads, unroll) 128x2, 256x1, 256x2, 256x4, 512x2
 constexpr int kAttrDefault = 1, kRepDefault = 2;
+constexpr int kAttrBoth = 2;           // force and energy in one pass
 int attr_variant_threads(int v);
 int rep_variant_threads(int v);
 int rep_variant_unroll(int v);

@@ -118,14 +118,16 @@ __global__ void pack_kernel(const KT *__restrict__ K, int64_t N, float4 *__restr
     flag_bad(bad, status);
 }
 
-// Resident CTAs the launch bounds ask for: three at 128 or 256 threads per
-// CTA (shared memory holds no more: registers <= 168 and <= 80), two at 512
-// (registers <= 64).
-constexpr int min_ctas(int nt) { return nt >= 512 ? 2 : 3; }
+// Resident CTAs the launch bounds ask for: what shared memory holds.  Three at
+// 128 or 256 threads per CTA (registers <= 168 and <= 80), two at 512 (registers
+// <= 64).  MODE 2 keeps a fourth sum (80 KB a CTA): two of any shape, which leaves
+// 255 and 128 registers (held to three CTAs' registers it spilled: 82750 samples
+// on 96^3 points 30.2 -> 17.6 ms at 128 threads, 20.4 -> 17.3 ms at 256).
+constexpr int min_ctas(int nt, int mode) { return nt >= 512 || mode == 2 ? 2 : 3; }
 
 // MODE 0: force, 1: energy, 2: both.
 template <int ACC, int MODE, int NT>
-__global__ void __launch_bounds__(NT, min_ctas(NT)) attraction_kernel(const AttrArgs a)
+__global__ void __launch_bounds__(NT, min_ctas(NT, MODE)) attraction_kernel(const AttrArgs a)
 {
     constexpr int kAcc = MODE == 2 ? kTile * 4 * 8 : kAccBytes;
     extern __shared__ __align__(128) float smem[];

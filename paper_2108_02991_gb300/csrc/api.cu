@@ -843,6 +843,9 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     cb.scale_dev = scale_dev;
     cb.eps = ctx->eps;
     cb.energy_blocks = at<double2>(ctx, P.o_eblocks);
+    // the directed sums' partials (15 MB and more) are free where the repulsion
+    // has totals or sums of its own
+    cb.few_blocks = totals || mesh_mode ? at<double2>(ctx, P.o_partr) : nullptr;
     if (mode == kEnergyKeep) {
         cb.attraction_only = true;
         LaunchScope ls(ctx, SPARKLING_KERNEL_COMBINE, st);

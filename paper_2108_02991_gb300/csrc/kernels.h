@@ -164,6 +164,7 @@ struct CombineArgs {
     double scale;         // G, A, R are multiplied by scale * (*scale_dev if set)
     const double *scale_dev;
     double2 *energy_blocks;  // energy mode: per-block (sum ea, sum er)
+    double2 *few_blocks;     // the same, of the few-samples form; null where part_r is in use
     double eps;           // regularisation: the N self pairs (|d| = eps each) leave F^r
 };
 

@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_few_kernel(const Combin
     }
     const double2 s = block_sum2(ea, er);
     if (threadIdx.x == 0)
-        c.energy_blocks[blockIdx.x] = s;
+        c.few_blocks[blockIdx.x] = s;
 }
 
 __global__ void __launch_bounds__(kEnergyThreads) energy_final_kernel(const double2 *blocks, int nb,
@@ -433,7 +433,8 @@ cudaError_t launch_attraction(const AttrArgs &a, int acc, int mode, int variant,
 }
 
 namespace {
-// Samples up to which a block of 256 / LANES samples is launched for each.
+// Samples up to which a block of 256 / LANES samples is launched for each (at
+// most 8192 blocks, whose energy sums take 128 KB).
 constexpr int64_t kFewSamples = 1 << 16;
 // Threads a sample of the slot sums: 0 (one thread a sample, grid-stride), 8, 32.
 int slot_lanes(const CombineArgs &c)
@@ -470,18 +471,12 @@ cudaError_t launch_combine(const CombineArgs &c, int out_dtype, int sms, cudaStr
     return cudaGetLastError();
 }
 
-// Block sums of an energy reduction of N samples, at most.
-int energy_blocks(int64_t N)
-{
-    const int64_t few = few_blocks(N < kFewSamples ? N : kFewSamples, 32);
-    const int64_t many = (N + kEnergyBlock - 1) / kEnergyBlock;
-    return (int)(few > many ? few : many);
-}
+int energy_blocks(int64_t N) { return (int)((N + kEnergyBlock - 1) / kEnergyBlock); }
 
 cudaError_t launch_combine_energy(const CombineArgs &c, double *out2, cudaStream_t st)
 {
-    const int lanes = slot_lanes(c);
-    const int nb = lanes ? few_blocks(c.N, lanes) : (int)((c.N + kEnergyBlock - 1) / kEnergyBlock);
+    const int lanes = c.few_blocks ? slot_lanes(c) : 0;
+    const int nb = lanes ? few_blocks(c.N, lanes) : energy_blocks(c.N);
     if (lanes == 8)
         energy_few_kernel<8><<<nb, kEnergyThreads, 0, st>>>(c);
     else if (lanes == 32)
@@ -490,7 +485,7 @@ cudaError_t launch_combine_energy(const CombineArgs &c, double *out2, cudaStream
         energy_block_kernel<<<nb, kEnergyThreads, 0, st>>>(c);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    energy_final_kernel<<<1, kEnergyThreads, 0, st>>>(c.energy_blocks, nb, c.N, c.eps, out2);
+    energy_final_kernel<<<1, kEnergyThreads, 0, st>>>(lanes ? c.few_blocks : c.energy_blocks, nb, c.N, c.eps, out2);
     return cudaGetLastError();
 }
 

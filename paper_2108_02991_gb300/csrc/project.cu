@@ -293,6 +293,9 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_batch_kernel(const
     }
 }
 
+// Violations of the result, a thread a sample whatever the shots' length: the
+// maxima are taken over all of them, so a block reduces once and not a shot at a
+// time.
 template <typename KT>
 __global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
 {
@@ -302,8 +305,13 @@ __global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
     for (int c = 0; c < 3; ++c) sp.pin[c] = p.pin[c];
     sp.pin_index = p.pin_index; sp.n_iter = p.n_iter; sp.check_every = 0;
     sp.viol = p.viol; sp.notconv = nullptr;
-    for (int64_t shot = blockIdx.x; shot < p.Nc; shot += gridDim.x)
-        record_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * (int64_t)p.Ns, sp);
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.Nc * p.Ns;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t shot = i / p.Ns;
+        sample_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * p.Ns, (int)(i - shot * p.Ns), sp, v);
+    }
+    reduce_violation(v, sp);
 }
 
 template <int CL> void *reg_fn(int dtype, int M)
@@ -445,7 +453,8 @@ cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, 
     void *args[] = {const_cast<ProjArgs *>(&p), const_cast<RegShape *>(&s)};
     cudaError_t e = launch_reg(fn, s, p.Nc, args, st);
     if (e != cudaSuccess || !p.viol) return e;
-    const unsigned g = (unsigned)(p.Nc < sms * 8 ? p.Nc : sms * 8);
+    const int64_t blocks = (p.Nc * p.Ns + 255) / 256;
+    const unsigned g = (unsigned)(blocks < sms * 8 ? blocks : sms * 8);
     if (dtype == 0) violation_kernel<float><<<g, 256, 0, st>>>(p);
     else violation_kernel<double><<<g, 256, 0, st>>>(p);
     return cudaGetLastError();

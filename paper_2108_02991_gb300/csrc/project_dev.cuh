@@ -399,32 +399,42 @@ __device__ void project_shot_mixed(const ArraysF &A, KT *Kshot, const ShotParams
 // Violations of an output shot already written to Kshot (device memory),
 // evaluated in FP64 and max-reduced into viol[4] (amplitude, slew, box, pin).
 template <typename KT>
-__device__ void record_violation(const KT *Kshot, const ShotParams &p)
+__device__ __forceinline__ void sample_violation(const KT *Kshot, int n, const ShotParams &p, double v[4])
 {
-    __syncthreads();
-    double v[4] = {0.0, 0.0, 0.0, 0.0}, unused = 0.0;
-    const int Ns = p.Ns;
-    for (int n = threadIdx.x; n < Ns; n += blockDim.x) {
-        double s0[3], s1[3], s2[3];
-        for (int c = 0; c < 3; ++c) {
-            s0[c] = (double)Kshot[3 * n + c];
-            v[2] = fmax(v[2], fabs(s0[c]) - p.box);
-            if (n == p.pin_index) v[3] = fmax(v[3], fabs(s0[c] - p.pin[c]));
-        }
-        if (n < Ns - 1) {
-            for (int c = 0; c < 3; ++c) s1[c] = (double)Kshot[3 * (n + 1) + c];
-            v[0] = fmax(v[0], norm3(s1[0] - s0[0], s1[1] - s0[1], s1[2] - s0[2]) - p.alpha);
-        }
-        if (n < Ns - 2) {
-            for (int c = 0; c < 3; ++c) s2[c] = (double)Kshot[3 * (n + 2) + c];
-            v[1] = fmax(v[1], norm3(s2[0] - 2.0 * s1[0] + s0[0], s2[1] - 2.0 * s1[1] + s0[1],
-                                    s2[2] - 2.0 * s1[2] + s0[2]) - p.beta);
-        }
+    double s0[3], s1[3], s2[3];
+    for (int c = 0; c < 3; ++c) {
+        s0[c] = (double)Kshot[3 * n + c];
+        v[2] = fmax(v[2], fabs(s0[c]) - p.box);
+        if (n == p.pin_index) v[3] = fmax(v[3], fabs(s0[c] - p.pin[c]));
     }
+    if (n < p.Ns - 1) {
+        for (int c = 0; c < 3; ++c) s1[c] = (double)Kshot[3 * (n + 1) + c];
+        v[0] = fmax(v[0], norm3(s1[0] - s0[0], s1[1] - s0[1], s1[2] - s0[2]) - p.alpha);
+    }
+    if (n < p.Ns - 2) {
+        for (int c = 0; c < 3; ++c) s2[c] = (double)Kshot[3 * (n + 2) + c];
+        v[1] = fmax(v[1], norm3(s2[0] - 2.0 * s1[0] + s0[0], s2[1] - 2.0 * s1[1] + s0[1],
+                                s2[2] - 2.0 * s1[2] + s0[2]) - p.beta);
+    }
+}
+
+// The threads' maxima, of one block, into p.viol.
+__device__ __forceinline__ void reduce_violation(double v[4], const ShotParams &p)
+{
+    double unused = 0.0;
     block_reduce(v, unused);
     if (threadIdx.x == 0)
         for (int e = 0; e < 4; ++e)
             atomicMax(&p.viol[e], (unsigned long long)__double_as_longlong(fmax(v[e], 0.0)));
+}
+
+template <typename KT>
+__device__ void record_violation(const KT *Kshot, const ShotParams &p)
+{
+    __syncthreads();
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int n = threadIdx.x; n < p.Ns; n += blockDim.x) sample_violation<KT>(Kshot, n, p, v);
+    reduce_violation(v, p);
     __syncthreads();
 }
 

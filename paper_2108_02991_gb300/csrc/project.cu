@@ -306,10 +306,15 @@ __global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
     sp.pin_index = p.pin_index; sp.n_iter = p.n_iter; sp.check_every = 0;
     sp.viol = p.viol; sp.notconv = nullptr;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.Nc * p.Ns;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t shot = i / p.Ns;
-        sample_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * p.Ns, (int)(i - shot * p.Ns), sp, v);
+    const unsigned int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    const int dshot = (int)(step / (unsigned int)p.Ns), dn = (int)(step % (unsigned int)p.Ns);
+    int64_t shot = first / (unsigned int)p.Ns;
+    int n = (int)(first % (unsigned int)p.Ns);
+    while (shot < p.Nc) {
+        sample_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * p.Ns, n, sp, v);
+        shot += dshot;
+        n += dn;
+        if (n >= p.Ns) { n -= p.Ns; ++shot; }
     }
     reduce_violation(v, sp);
 }
@@ -453,10 +458,13 @@ cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, 
     void *args[] = {const_cast<ProjArgs *>(&p), const_cast<RegShape *>(&s)};
     cudaError_t e = launch_reg(fn, s, p.Nc, args, st);
     if (e != cudaSuccess || !p.viol) return e;
-    const int64_t blocks = (p.Nc * p.Ns + 255) / 256;
-    const unsigned g = (unsigned)(blocks < sms * 8 ? blocks : sms * 8);
-    if (dtype == 0) violation_kernel<float><<<g, 256, 0, st>>>(p);
-    else violation_kernel<double><<<g, 256, 0, st>>>(p);
+    // a block an SM (a sample takes ~4 us of FP64 latency); more, for the width,
+    // only with two samples a thread, as a block's reduction costs about one
+    const int64_t total = p.Nc * p.Ns, one = (total + 255) / 256, two = (total + 511) / 512;
+    int64_t g = two < (int64_t)sms * 4 ? two : (int64_t)sms * 4;
+    if (g < sms) g = one < sms ? one : sms;
+    if (dtype == 0) violation_kernel<float><<<(unsigned)g, 256, 0, st>>>(p);
+    else violation_kernel<double><<<(unsigned)g, 256, 0, st>>>(p);
     return cudaGetLastError();
 }
 

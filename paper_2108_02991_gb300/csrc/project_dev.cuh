@@ -418,14 +418,17 @@ __device__ __forceinline__ void sample_violation(const KT *Kshot, int n, const S
     }
 }
 
-// The threads' maxima, of one block, into p.viol.
+// The threads' maxima, of one block, into p.viol (where they are larger: the
+// blocks' atomics meet at four words).
 __device__ __forceinline__ void reduce_violation(double v[4], const ShotParams &p)
 {
     double unused = 0.0;
     block_reduce(v, unused);
     if (threadIdx.x == 0)
-        for (int e = 0; e < 4; ++e)
-            atomicMax(&p.viol[e], (unsigned long long)__double_as_longlong(fmax(v[e], 0.0)));
+        for (int e = 0; e < 4; ++e) {
+            const unsigned long long bits = (unsigned long long)__double_as_longlong(fmax(v[e], 0.0));
+            if (bits > *(volatile unsigned long long *)&p.viol[e]) atomicMax(&p.viol[e], bits);
+        }
 }
 
 template <typename KT>

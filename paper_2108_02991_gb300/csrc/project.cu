@@ -212,7 +212,8 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_reg_kernel(const P
     __shared__ typename RegEdges<R, M, CL>::Shared shared;
     RegEdges<R, M, CL> edges(&shared, shape);
     RegShot sh;
-    sh.Ns = p.Ns; sh.n_iter = p.n_iter; sh.pin_index = p.pin_index;
+    // a lone sample has no rows: its projection is the clip (or the pin)
+    sh.Ns = p.Ns; sh.n_iter = p.Ns > 1 ? p.n_iter : 0; sh.pin_index = p.pin_index;
     sh.alpha = p.alpha; sh.beta = p.beta; sh.box = p.box;
     for (int c = 0; c < 3; ++c) sh.pin[c] = p.pin[c];
     KT *K = static_cast<KT *>(p.K);
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_batch_kernel(const
         const EngineTraj &tr = e.traj[lo];
         if (e.done[lo] < (unsigned int)tr.n_pair_items) continue;   // the whole cluster alike
         RegShot sh;
-        sh.Ns = Ns; sh.n_iter = tr.n_iter; sh.pin_index = tr.pin_index;
+        sh.Ns = Ns; sh.n_iter = Ns > 1 ? tr.n_iter : 0; sh.pin_index = tr.pin_index;
         sh.alpha = tr.alpha; sh.beta = tr.beta; sh.box = tr.box;
         for (int c = 0; c < 3; ++c) sh.pin[c] = tr.pin[c];
         float *K = static_cast<float *>(e.K) + 3 * shot * (int64_t)Ns;
@@ -362,13 +363,13 @@ bool reg_halo_shape(int Ns, int M, int C, RegShape &s)
     return s.threads <= reg_max_threads(M) && s.halo >= 8 && Ns - (C - 1) * s.own >= s.halo;
 }
 
-// Time of 100 iterations (us) where every CTA has an SM to itself: a chain's
-// latency, or the issue of the SM's warps (FP64: of its FP64 pipe); ~0.5 us a
-// cluster barrier, of which a shape with halos has two a copy.  Fitted to
-// shots of 64 .. 2560 samples.
-double reg_time(bool fp64, const RegShape &s)
+// Time of 100 iterations (us) where an SM has `load` CTAs: a chain's latency,
+// or the issue of the SM's warps (FP64: of its FP64 pipe); ~0.5 us a cluster
+// barrier, of which a shape with halos has two a copy.  Fitted to shots of
+// 64 .. 2560 samples, load 1.
+double reg_time(bool fp64, const RegShape &s, double load = 1.0)
 {
-    const int w = s.threads / 32;
+    const double w = load * (s.threads / 32);
     const bool one = s.per_thread == 1;
     const double chain = fp64 ? (one ? 310.0 : 550.0) : one ? 88.0 : 108.0;
     const double warp = fp64 ? (one ? 72.0 : 122.0) : one ? 14.0 : 19.0;
@@ -385,9 +386,10 @@ double reg_time(bool fp64, const RegShape &s)
 // 448).  Shots of up to 128 samples are bound by the latency of one warp's
 // chain: M = 1 (32 x 64: 86 against 107 us, then too).
 // FP64: bound by the FP64 pipe, which every warp of an SM shares.  M = 1 costs
-// ~10 % more operations but pads less and has the shorter chain; it is taken
-// where the shots do not fill the GPU (37 x 129: 379 against 531 us; 300 x
-// 700: 2.80 against 2.53 ms).  One CTA up to 1024 samples (a cluster barrier
+// ~10 % more operations but pads less and has the shorter chain: the times
+// above decide, with the CTAs that fall to an SM (37 x 129: 379 against 531 us;
+// 300 x 700: 2.80 against 2.53 ms; 20000 x 32, half a warp at M = 2: 7.6
+// against 15.0 ms; 300 x 96: 428 against 561 us).  One CTA up to 1024 samples (a cluster barrier
 // costs ~0.4 us: 300 x 700 as 2 CTAs takes 2.79 ms), else at most 256 threads.
 // Few shots (`halos`; every CTA with an SM to itself): more, smaller CTAs a
 // shot with halos, as the times above say.  FP64 8 x 1000 1891 -> 410 us, 20 x
@@ -396,12 +398,22 @@ RegShape project_reg_shape(int dtype, int64_t Nc, int Ns, int sms, bool halos)
 {
     RegShape s;
     const bool fp64 = dtype != 0;
-    s.per_thread = fp64 ? (Nc <= sms && Ns <= 256 ? 1 : 2) : (Ns <= 128 ? 1 : 2);
     const int one = fp64 ? 1024 : 512;            // samples a single CTA takes
     s.ctas = Ns <= one ? 1 : (Ns + 511) / 512;
     if (s.ctas > kRegMaxCtas) s.ctas = kRegMaxCtas;
-    const int per = s.ctas * s.per_thread;
-    s.threads = ((Ns + per - 1) / per + 31) / 32 * 32;
+    auto with = [&](int M) {
+        RegShape t = s;
+        t.per_thread = M;
+        const int per = s.ctas * M;
+        t.threads = ((Ns + per - 1) / per + 31) / 32 * 32;
+        return t;
+    };
+    if (fp64 && s.ctas == 1 && Ns <= reg_max_threads(1)) {
+        const double load = (double)((Nc + sms - 1) / sms);
+        s = reg_time(true, with(1), load) <= reg_time(true, with(2), load) ? with(1) : with(2);
+    } else {
+        s = with(!fp64 && Ns <= 128 ? 1 : 2);
+    }
     if (!halos) return s;
     double best = 0.95 * reg_time(fp64, s);
     for (int M = 1; M <= 2; ++M)

@@ -80,3 +80,41 @@ def test_violations_cost_little(sp, ctx, dt):
     most three times the projection alone (a block a shot took ten times)."""
     assert (project_ms(sp, ctx, 20000, 2, dt, 1, viol=True) <
             3.0 * project_ms(sp, ctx, 20000, 2, dt, 1) + 0.02)
+
+
+def check(sp, ctx, Nc, Ns, dt, n_iter, pin_index=-1):
+    K = shots(Nc, Ns, dt)
+    a, b = radii(Ns)
+    ref = oracle.project(K.astype(np.float64), Nc, Ns, a, b, box=0.5, pin_index=pin_index, n_iter=n_iter)
+    ref = ref[0] if isinstance(ref, tuple) else ref
+    Kd = torch.from_numpy(K).cuda()
+    sp.sparkling_project(ctx, Kd, Nc, Ns, sp.make_proj(a, b, 0.5, n_iter, pin_index))
+    if dt == np.float64:
+        np.testing.assert_allclose(Kd.cpu().numpy(), ref, rtol=0, atol=1e-11)
+    else:
+        np.testing.assert_allclose(Kd.cpu().numpy(), ref.astype(np.float32), rtol=0, atol=PROJ_F32_ROUND)
+
+
+@pytest.mark.parametrize("Nc,Ns", [(400, 1), (400, 2), (153, 31), (700, 32), (700, 33), (300, 65), (300, 96),
+                                   (160, 160), (153, 255), (153, 257), (160, 767), (153, 769)])
+def test_more_fp64_shots_than_sms(sp, ctx, Nc, Ns):
+    check(sp, ctx, Nc, Ns, np.float64, 25, pin_index=Ns - 1)
+
+
+@pytest.mark.parametrize("n_iter", [0, 1, 100])
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+def test_lone_samples_are_clipped(sp, ctx, dt, n_iter):
+    K = torch.from_numpy(shots(500, 1, dt)).cuda()
+    want = K.clamp(-0.5, 0.5)
+    sp.sparkling_project(ctx, K, 500, 1, sp.make_proj(*radii(1), 0.5, n_iter))
+    assert torch.equal(K, want)
+
+
+def test_fp64_times_follow_the_samples(sp, ctx):
+    """Bound by the FP64 pipe, which half a warp occupies like a whole one:
+    shots of 32 samples take one warp of one sample a thread (72 units an
+    iteration) where 33 samples take one of two (122), expected 0.6, gate 0.8
+    (it was 1.0); lone samples have no iteration to do."""
+    t = {n: project_ms(sp, ctx, 20000, n, np.float64, 100) for n in (1, 2, 32, 33)}
+    assert t[32] < 0.8 * t[33]
+    assert t[1] < 0.2 * t[2]

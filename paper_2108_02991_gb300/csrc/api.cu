@@ -28,8 +28,11 @@ using namespace sparkling;
 constexpr int64_t kStepEngineMin = (int64_t)1 << 22;
 
 // Up to this many samples the repulsion runs directed over the whole GPU
-// (repulsion_small.cu) instead of on pairs of 1024-sample tiles.
-constexpr int64_t kSmallRepulsion = 20480;
+// (repulsion_small.cu) instead of on pairs of 1024-sample tiles.  Gradient /
+// energy, directed against symmetric: 10240 samples 62 / 66 us against 78 / 69,
+// 11000 71 / 76 against 88 / 69, 12288 87 / 96 against 78 / 69, 20480 189 / 176
+// against 137 / 116.
+constexpr int64_t kSmallRepulsion = 11 * 1024;
 
 struct sparkling_ctx {
     int device = 0;
@@ -709,6 +712,30 @@ int ensure_mesh(sparkling_ctx *ctx, cudaStream_t st)
     return SPARKLING_OK;
 }
 
+// Tiles from which the tuner chooses the symmetric kernel's shape for the force.
+constexpr int64_t kSymTuneTiles = 64;
+
+// Shape of the symmetric kernel.  With few waves of tile pairs their number
+// decides, not the rate a tuner would find at another size: a CTA's pairs follow
+// one another, and one takes 80 us (shape 2) or 78 us (shape 3) where an SM has one
+// CTA and 70 / 60 us more for every other CTA on it (gradient: 300 pairs 151 /
+// 138 us, 465 pairs 291 / 390 us, of which shape 2 runs 304 and shape 3 456 at once).
+int sym_shape(const sparkling_ctx *ctx, int64_t tiles, bool energy)
+{
+    if (ctx->pin_sym) return ctx->sym_choice;
+    if (energy) return kSymEnergy;
+    if (ctx->autotune && tiles < kSymTuneTiles) {
+        const int64_t units = tri_count(tiles);
+        auto time = [&](int v, double one, double other) {
+            const int64_t ctas = std::min<int64_t>(units, (int64_t)ctx->sms * ctx->occ_sym[0][v]);
+            const int64_t on_sm = (ctas + ctx->sms - 1) / ctx->sms;
+            return (double)((units + ctas - 1) / ctas) * (one + other * (double)(on_sm - 1));
+        };
+        return time(2, 80.0, 70.0) < time(3, 78.0, 59.5) ? 2 : 3;
+    }
+    return ctx->sym_choice < 0 ? kSymDefault : ctx->sym_choice;
+}
+
 // The repulsion sums of the packed samples: into the totals racc (few samples,
 // symmetric kernel), into r_direct (mesh; set here) or into ra.part (directed).
 int run_repulsion(sparkling_ctx *ctx, PairPlan &P, const float4 *pos, const RepArgs &ra, int acc,
@@ -745,7 +772,7 @@ int run_repulsion(sparkling_ctx *ctx, PairPlan &P, const float4 *pos, const RepA
         // every unordered pair once, exact fixed-point totals
         SymArgs sa{};
         sa.pos = pos; sa.N = P.N; sa.tiles = P.tiles;
-        const int sv = ctx->sym_choice < 0 ? kSymDefault : ctx->sym_choice;
+        const int sv = sym_shape(ctx, P.tiles, energy);
         sa.ctas = (int64_t)ctx->sms * ctx->occ_sym[energy ? 1 : 0][sv];
         sa.acc = racc; sa.status = ctx->d_status; sa.eps2 = ra.eps2;
         CK(launch_repulsion_sym(sa, energy, sv, st));
@@ -806,7 +833,8 @@ int run_pairs(sparkling_ctx *ctx, const void *K, int K_dtype, const sparkling_gr
     ra.eps2 = aa.eps2;
     const bool need_a = !field_mode && !A_kept && attr_choice_of(ctx, acc, P.gxp) < 0,
                need_r = !mesh_mode && !small && !ctx->rep_symmetric && ctx->rep_choice[rep_acc(acc)] < 0,
-               need_s = !mesh_mode && !small && ctx->rep_symmetric && ctx->sym_choice < 0;
+               need_s = !mesh_mode && !small && ctx->rep_symmetric && ctx->sym_choice < 0 &&
+                        P.tiles >= kSymTuneTiles;
     if (ctx->autotune && (need_a || need_r || need_s)) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         CK(cudaStreamIsCapturing(st, &cap));

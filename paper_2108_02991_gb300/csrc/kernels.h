@@ -205,6 +205,10 @@ cudaError_t launch_combine(const CombineArgs &c, int out_dtype, int sms, cudaStr
 // per lane), 2 sources paired (3).
 constexpr int kSymVariants = 4;
 constexpr int kSymDefault = 3;        // shape used where nothing was tuned or pinned
+// Shape of the energy unless one is pinned: the tuner times the force, which
+// takes shape 3 more often (energy, shapes 2 / 3: 20480 samples 116 / 122 us,
+// 65536 675 / 735, 100000 1517 / 1673).
+constexpr int kSymEnergy = 2;
 int sym_variant_sources(int v);
 bool sym_variant_source_paired(int v);
 int sym_variant_threads(int v);

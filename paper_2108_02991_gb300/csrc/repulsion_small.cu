@@ -10,9 +10,9 @@
 //
 // Bound: latency up to ~4000 samples, FP32 issue (11.5 instructions a directed
 // pair) above.  Measured (gradient; the call's scope, uniform samples): 1024
-// samples 8.1 us against 78 with the symmetric kernel, 4773 20 against 209, 8192
-// 43 against 199, 12288 88 against 199, 16384 128 against 137, 20480 189 against
-// 200, 24576 260 against 200; the rule of the dispatch (api.cu) follows from these.
+// samples 8.2 us against 78 with the symmetric kernel, 4096 16 against 77, 8192
+// 43 against 78, 11000 71 against 88, 12288 87 against 78, 16384 128 against 78;
+// the rule of the dispatch (api.cu) follows from these.
 #include <cuda_runtime.h>
 #include <cstdint>
 

@@ -306,7 +306,8 @@ __device__ __forceinline__ void r_update(const VecDf &z, Df r, float r2, const f
     const Df g = r_mul_raw(r, Df{x, x * (e * fmaf(0.375f, e, 0.5f))});
     const Df s = df_renorm(1.f, -g.h);          // g <= 1 up to rounding
     Df f = df_renorm(s.h, __fsub_rn(s.l, g.l));
-    // inside the ball (or no such row): 0; NaN goes on, and stays
+    // inside the ball (or no such row): 0; NaN goes on, and stays.  r2 lies a
+    // little below the radius squared: near it the sign of f decides, on both words
     if (!exists || zz.h <= r2 || f.h < 0.f) f = {0.f, 0.f};
     const FactorDf a(r_mul(f, Df{m.x, m.y})), b(r_mul(f, Df{m.z, m.w}));
     y = v_norm(v_sub_raw(v_mul_raw(z, a), w));
@@ -329,9 +330,11 @@ __device__ __forceinline__ float4 momentum_of(const MomentumTables &m, int it, b
 __device__ __forceinline__ double factor_of(double f) { return f; }
 __device__ __forceinline__ FactorDf factor_of(Df f) { return FactorDf(f); }
 
-// Squared radius as the type the comparison takes.
+// Squared radius as the type the comparison takes; two floats: the square of the
+// leading word less 2^-20 of it, so that a row below it is inside for certain
+// (infinity stays).
 __device__ __forceinline__ double r_square(double r) { return r * r; }
-__device__ __forceinline__ float r_square(Df r) { return r.h * r.h; }
+__device__ __forceinline__ float r_square(Df r) { return r.h * r.h * (1.f - 1.f / (1 << 20)); }
 
 // ---- the projection ---------------------------------------------------------
 

@@ -263,14 +263,20 @@ __device__ __forceinline__ void r_update(const VecD &z, double r, double r2, con
 {
     const double zz = fma(z.x, z.x, fma(z.y, z.y, z.z * z.z));
     double f = 0.0;
-    // both non-negative: integer comparison (NaN compares above)
-    const bool on = exists && __double_as_longlong(zz) > __double_as_longlong(r2);
+    // both non-negative: comparison as integers, unsigned (a NaN of either sign
+    // compares above)
+    const unsigned long long zb = (unsigned long long)__double_as_longlong(zz);
+    const bool on = exists && zb > (unsigned long long)__double_as_longlong(r2);
     if (on) {
-        double x;
-        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(zz));
-        const double e = fma(-zz * x, x, 1.0);
-        x = fma(x * e, fma(0.375, e, 0.5), x);
-        f = fma(-r, x, 1.0);
+        if ((unsigned int)(zb >> 32) - 0x00100000u < 0x7fe00000u) {
+            double x;
+            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(zz));
+            const double e = fma(-zz * x, x, 1.0);
+            x = fma(x * e, fma(0.375, e, 0.5), x);
+            f = fma(-r, x, 1.0);
+        } else if (zz == zz) {                 // subnormal or infinite
+            f = fma(-r, rsqrt(zz), 1.0);
+        }                                      // NaN stays in its component
     }
     auto row = [&](double zc, double &qc, double &yc) {
         const double qn = on ? zc * f : 0.0;
@@ -306,9 +312,10 @@ __device__ __forceinline__ void r_update(const VecDf &z, Df r, float r2, const f
     const Df g = r_mul_raw(r, Df{x, x * (e * fmaf(0.375f, e, 0.5f))});
     const Df s = df_renorm(1.f, -g.h);          // g <= 1 up to rounding
     Df f = df_renorm(s.h, __fsub_rn(s.l, g.l));
-    // inside the ball (or no such row): 0; NaN goes on, and stays.  r2 lies a
-    // little below the radius squared: near it the sign of f decides, on both words
-    if (!exists || zz.h <= r2 || f.h < 0.f) f = {0.f, 0.f};
+    // inside the ball (or no such row): 0, and for NaN, which stays in its
+    // component.  r2 lies a little below the radius squared: near it the sign of f
+    // decides, on both words
+    if (!exists || zz.h <= r2 || !(f.h >= 0.f)) f = {0.f, 0.f};
     const FactorDf a(r_mul(f, Df{m.x, m.y})), b(r_mul(f, Df{m.z, m.w}));
     y = v_norm(v_sub_raw(v_mul_raw(z, a), w));
     w = v_mul(z, b);

@@ -51,3 +51,52 @@ def test_a_row_at_its_radius(sp, ctx, c, d, rows, dt):
     out = project(sp, ctx, K, 3, Ns, *r, 0.5, 300)
     assert d < 0 or abs(ref[0, 1]) > 0.1 * c * d      # away from or towards the last sample
     np.testing.assert_allclose(out[0::Ns], ref[0::Ns], rtol=2.0 ** -23, atol=c * 2.0 ** -44)
+
+
+def walk(Ns, seed=0):
+    return np.cumsum(np.random.default_rng(seed).normal(scale=0.02, size=(2, Ns, 3)), axis=1).reshape(-1, 3)
+
+
+@pytest.mark.parametrize("Ns", [40, 600, 1100])
+@pytest.mark.parametrize("e,tol", [(400, 1e-11), (-400, 1e-11), (-520, 1e-4)])
+def test_fp64_samples_of_any_scale(sp, ctx, Ns, e, tol):
+    """The projection of s K onto s times the set is s times the projection.  At
+    2^-520 the squares are subnormal (2^-1054 and less: 20 bits and less of the
+    smallest, 1e-4 of a dual)."""
+    s = 2.0 ** e
+    a, b = 1.0 / (2 * Ns), 1.0 / (8 * Ns * Ns)
+    if e == -520:
+        a, b = 0.01, 0.02                     # squares of 2^-1053 and up
+    K = walk(Ns)
+    ref = oracle.project(K, 2, Ns, a, b, n_iter=30)
+    out = project(sp, ctx, K * s, 2, Ns, a * s, b * s, 0.5 * s, 30)
+    np.testing.assert_allclose(out / s, ref, rtol=0, atol=tol)
+
+
+def test_fp64_samples_whose_squares_overflow(sp, ctx):
+    """1/|z| is 0 then: the row keeps its length, and stays finite."""
+    out = project(sp, ctx, walk(40) * 2.0 ** 530, 2, 40, 2.0 ** 505, 2.0 ** 505, 2.0 ** 529, 30)
+    assert np.isfinite(out).all() and np.abs(out).max() <= 2.0 ** 529
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("n_iter", [0, 1, 3, 40])
+def test_not_a_number_spreads_as_the_rows_do(sp, ctx, dt, n_iter, sign):
+    """Two samples an iteration to either side, in all components, of that shot."""
+    K = walk(200).astype(dt)
+    K[70, 1] = np.copysign(np.nan, sign)
+    out = project(sp, ctx, K, 2, 200, 0.01, 1e-4, 0.5, n_iter)
+    want = oracle.project(K.astype(np.float64), 2, 200, 0.01, 1e-4, n_iter=n_iter)
+    np.testing.assert_array_equal(np.isnan(out), np.isnan(want))
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+def test_infinities_are_clipped(sp, ctx, dt):
+    K = walk(200).astype(dt)
+    K[70, 1], K[71, 2] = np.inf, -np.inf
+    out = project(sp, ctx, K, 2, 200, 0.01, 1e-4, 0.5, 20)
+    big = K.copy()
+    big[70, 1], big[71, 2] = 1e18, -1e18      # beyond any dual's reach
+    want = oracle.project(big.astype(np.float64), 2, 200, 0.01, 1e-4, n_iter=20)
+    np.testing.assert_allclose(out, want, rtol=0, atol=1e-11 if dt == np.float64 else 2.0 ** -24)

@@ -22,7 +22,7 @@ grid 256^3 = 16,777,216 points (the ~1e7-sample configuration).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                   [--workload hr|diff|medium|small|tiny|batched]
-                  [--acc kahan|fp64|fp64pair] [--projection fp64|mixed]
+                  [--acc kahan|fp64|fp64pair] [--projection default|fp64|mixed]
 
 Under torchrun (N > 1) every rank runs an independent problem instance of
 the same size (its own seed) on its own GPU: the trajectories are
@@ -72,9 +72,9 @@ def parse_args(argv=None):
     ap.add_argument("--two-launches", action="store_true",
                     help="batched step: the symmetric repulsion in its own kernel ahead of the "
                          "engine instead of as items of the engine's work list (one launch)")
-    ap.add_argument("--projection", choices=("fp64", "mixed"), default="fp64",
-                    help="projection arithmetic: the default (FP64, two-float sums for FP32 samples) or "
-                         "mixed (an FP32 iteration is allowed)")
+    ap.add_argument("--projection", choices=("default", "fp64", "mixed"), default="default",
+                    help="projection arithmetic: the default (FP64, two-float sums for FP32 samples), "
+                         "fp64 for every sample type, or mixed (an FP32 iteration is allowed)")
     ap.add_argument("--shot-stride", type=int, default=1,
                     help="keep every S-th shot of the workload (same density): a smaller launch "
                          "of the same kernels, e.g. for a profiler capture")
@@ -496,8 +496,8 @@ def run_ours(args):
     if args.shape_repulsion >= 0:
         sp.sparkling_set_shape(ctx, "repulsion", args.shape_repulsion)
     sp.sparkling_set_step_path(ctx, args.path)
-    sp.sparkling_set_projection(ctx, sp.PROJECTION_MIXED if args.projection == "mixed"
-                                else sp.PROJECTION_FP64)
+    sp.sparkling_set_projection(ctx, {"default": sp.PROJECTION_DEFAULT, "fp64": sp.PROJECTION_FP64,
+                                      "mixed": sp.PROJECTION_MIXED}[args.projection])
     stream = torch.cuda.current_stream(dev)
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
     field_build_ms = None
@@ -671,8 +671,9 @@ def run_ours(args):
 
     if rank == 0:
         p0 = w.probs[0]
-        proj_form = ("mixed FP32/FP64 projection" if args.projection == "mixed"
-                     else "FP64 projection step, duals and primal in two-float sums (48 bits)")
+        proj_form = {"default": "FP64 projection step, duals and primal in two-float sums (48 bits)",
+                     "fp64": "FP64 projection",
+                     "mixed": "mixed FP32/FP64 projection"}[args.projection]
         acc_form = {"kahan": "compensated-f32 per-target sums",
                     "fp64": "f64 per-target sums of f32 row sums",
                     "fp64pair": "every attraction pair term added in f64"}[args.acc]

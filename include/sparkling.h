@@ -133,7 +133,8 @@ typedef struct sparkling_proj {
 #define SPARKLING_KERNEL_COUNT 8
 
 /* Arithmetic of the projection (sparkling_set_projection). */
-#define SPARKLING_PROJECTION_FP64 0    /* FP64, or 48-bit two-float sums where the result is FP32 (default) */
+#define SPARKLING_PROJECTION_DEFAULT -1 /* FP64, or 48-bit two-float sums where the result is FP32 */
+#define SPARKLING_PROJECTION_FP64 0    /* FP64 for every K dtype */
 #define SPARKLING_PROJECTION_MIXED 1   /* FP32 K, fixed n_iter: FP32 iteration allowed */
 
 /* How sparkling_step runs its device work (sparkling_set_step_path). */
@@ -427,12 +428,14 @@ SPARKLING_API int sparkling_set_regularisation(sparkling_ctx *ctx, double eps);
 
 /* Arithmetic of the context's projections (sparkling_project, sparkling_step,
  * sparkling_step_host, sparkling_step_batched, the driver).
- *   SPARKLING_PROJECTION_FP64 (default): the dual FISTA iteration, the primal
- *     map and the step in FP64; the result is rounded to K_dtype once.  For
- *     FP32 K with a fixed n_iter <= 4096, Ns <= 8192 and alpha, beta (or inf),
- *     box and pin in [2^-40, 2^40], the duals and the primal map are carried
- *     as unevaluated sums of two floats (48 bits; the step k = K - eta G in
- *     FP64) -- the FP32 result is the FP64 one up to its last rounding.
+ *   SPARKLING_PROJECTION_DEFAULT (a new context's): the dual FISTA iteration,
+ *     the primal map and the step in FP64; the result is rounded to K_dtype
+ *     once.  For FP32 K with a fixed n_iter <= 4096, Ns <= 8192 and alpha, beta
+ *     (or inf), box and pin in [2^-40, 2^40], the duals and the primal map are
+ *     carried as unevaluated sums of two floats (48 bits; the step k = K - eta G
+ *     in FP64) -- the FP32 result is the FP64 one up to its last rounding, in an
+ *     eighth of the time and less.
+ *   SPARKLING_PROJECTION_FP64: the same in FP64 for every K dtype and size.
  *   SPARKLING_PROJECTION_MIXED: lets FP32 K with a fixed n_iter iterate in
  *     FP32 on the displacement e = s - k and the duals (D1 k, D2 k and the box
  *     and pin offsets formed once per shot in FP64, the output k + e in FP64)

@@ -19,7 +19,7 @@ OK, E_INVAL, E_NOMEM, E_CUDA, E_NONFINITE, E_TIMEOUT, E_NOTCONV, E_IO, E_RANGE =
 F32, F64 = 0, 1
 ACC_KAHAN32, ACC_FP64, ACC_FP64_PAIR = 0, 1, 2
 KERNEL_NAMES = ("pack", "attraction", "repulsion", "combine", "project", "engine", "driver", "step")
-PROJECTION_FP64, PROJECTION_MIXED = 0, 1
+PROJECTION_DEFAULT, PROJECTION_FP64, PROJECTION_MIXED = -1, 0, 1
 BATCH_GRAPH = 1
 BATCH_TWO_LAUNCHES = 2
 STEP_AUTO, STEP_KERNELS, STEP_ENGINE = 0, 1, 2
@@ -463,8 +463,9 @@ def sparkling_set_attraction(ctx: Context, mode: int) -> None:
 
 
 def sparkling_set_projection(ctx: Context, mode: int) -> None:
-    """PROJECTION_FP64 (default: FP64 iteration, or 48-bit two-float sums for
-    FP32 K) or PROJECTION_MIXED (FP32 K: an FP32 iteration is allowed)."""
+    """PROJECTION_DEFAULT (FP64 iteration, or 48-bit two-float sums for FP32 K),
+    PROJECTION_FP64 (FP64 for every K) or PROJECTION_MIXED (FP32 K: an FP32
+    iteration is allowed)."""
     _check(ctx, lib().sparkling_set_projection(ctx.handle, int(mode)))
 
 

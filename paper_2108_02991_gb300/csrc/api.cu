@@ -41,7 +41,7 @@ struct sparkling_ctx {
     int *d_status = nullptr;    // device control block (DevCtl): status word, wait budget
     long long wait_cycles = kWaitCycles;   // budget of the kernels' bounded waits
     size_t mem_limit = 0;       // cap on the context's device allocations (0: none)
-    int proj_mode = SPARKLING_PROJECTION_FP64;
+    int proj_mode = SPARKLING_PROJECTION_DEFAULT;
     int step_path = SPARKLING_STEP_AUTO;
     double *d_small = nullptr;  // [0..1] energy, [2..5] violation bits, [6] notconv (int)
     void *d_mom = nullptr;      // momentum factors of the projection (MomentumTables)
@@ -936,6 +936,13 @@ int common_checks(sparkling_ctx *ctx, const void *K, int K_dtype, int64_t N, con
     return SPARKLING_OK;
 }
 
+// Whether the context leaves the samples' projection to the register form: FP64
+// asked for means FP64 for FP32 samples too.
+bool reg_allowed(const sparkling_ctx *ctx, int K_dtype)
+{
+    return K_dtype != SPARKLING_F32 || ctx->proj_mode != SPARKLING_PROJECTION_FP64;
+}
+
 // Launch shape of the projection: one CTA per shot up to one wave; the
 // per-CTA state goes to the workspace when it does not fit in shared memory.
 struct ProjPlan {
@@ -949,7 +956,8 @@ int plan_project(sparkling_ctx *ctx, int K_dtype, int64_t Nc, int64_t Ns, const 
                  Carve &cv, ProjPlan &L)
 {
     const int ns = (int)Ns;
-    if (project_reg_applies(K_dtype, ns, pr->alpha, pr->beta, pr->box, pr->tol, pr->pin,
+    if (reg_allowed(ctx, K_dtype) &&
+        project_reg_applies(K_dtype, ns, pr->alpha, pr->beta, pr->box, pr->tol, pr->pin,
                             pr->pin_index, pr->n_iter)) {
         L.reg = project_reg_shape(K_dtype, Nc, ns, ctx->sms, true);
         return SPARKLING_OK;
@@ -1828,7 +1836,7 @@ SPARKLING_API int sparkling_step_batched(sparkling_ctx *ctx, int32_t B, const in
     // the engine they cost 24 of 248 ms on 16 trajectories (2.4e6 samples),
     // after it 5.  FP64 samples keep them in the engine, whose pair items
     // leave the FP64 pipe idle.
-    bool split_proj = K_dtype == SPARKLING_F32;
+    bool split_proj = K_dtype == SPARKLING_F32 && reg_allowed(ctx, K_dtype);
     for (int t = 0; t < B && split_proj; ++t)
         split_proj = project_reg_applies(K_dtype, Ns, proj[t].alpha, proj[t].beta, proj[t].box, 0.0,
                                          proj[t].pin, proj[t].pin_index, proj[t].n_iter);
@@ -2097,8 +2105,9 @@ SPARKLING_API int sparkling_set_shape(sparkling_ctx *ctx, int kernel, int varian
 SPARKLING_API int sparkling_set_projection(sparkling_ctx *ctx, int mode)
 {
     if (!ctx) return fail(nullptr, SPARKLING_E_INVAL, "ctx is NULL");
-    if (mode != SPARKLING_PROJECTION_FP64 && mode != SPARKLING_PROJECTION_MIXED)
-        return fail(ctx, SPARKLING_E_INVAL, "projection mode %d is not FP64/MIXED", mode);
+    if (mode != SPARKLING_PROJECTION_DEFAULT && mode != SPARKLING_PROJECTION_FP64 &&
+        mode != SPARKLING_PROJECTION_MIXED)
+        return fail(ctx, SPARKLING_E_INVAL, "projection mode %d is not DEFAULT/FP64/MIXED", mode);
     ctx->proj_mode = mode;
     return SPARKLING_OK;
 }

@@ -1267,7 +1267,7 @@ int batch_engine(sparkling_ctx *ctx, void *K, int K_dtype, int acc, int variant,
     e.wait_scale = b.wait_scale;
     e.n_attr = b.n_attr;
     e.n_sym = b.n_sym;
-    e.gstate = b.proj_in_smem ? nullptr : at<double>(ctx, b.o_gstate);
+    e.gstate = b.proj_in_smem || b.split_proj ? nullptr : at<double>(ctx, b.o_gstate);
     e.status = ctx->d_status;
     e.eps2 = eps2_of(ctx);
     e.racc = b.sym || b.one_launch ? at<unsigned long long>(ctx, b.o_racc) : nullptr;
@@ -1869,7 +1869,9 @@ SPARKLING_API int sparkling_step_batched(sparkling_ctx *ctx, int32_t B, const in
         for (int t = 0; t < B; ++t) parts += (int64_t)b.traj[t].tiles * b.traj[t].slots;
         b.o_part = cv.take((size_t)parts * kTile * sizeof(dacc4));
         b.proj_in_smem = project_state_bytes(Ns) <= engine_proj_smem_limit();
-        if (!b.proj_in_smem) b.o_gstate = cv.take((size_t)ctas * project_state_bytes(Ns));
+        // the state of the list's projection items, if it has any
+        if (!b.proj_in_smem && !split_proj)
+            b.o_gstate = cv.take((size_t)ctas * project_state_bytes(Ns));
         if (b.sym || b.one_launch)
             b.o_racc = cv.take((size_t)off[B] * 3 * sizeof(unsigned long long));
         if (b.sym) {

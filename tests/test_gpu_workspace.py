@@ -46,3 +46,20 @@ def test_few_samples_ask_for_samples_and_totals(sp, tiles):
                  lambda c, N: sp.sparkling_grad(c, samples(N), g)):
         more = asked(sp, lambda c: call(c, hi)) - asked(sp, lambda c: call(c, lo))
         assert more <= (hi - lo) * 40 + 3 * 256
+
+
+def test_projections_in_a_second_launch_ask_for_no_state(sp):
+    """FP32 trajectories of 2560 samples a shot: as items (FP64 asked for) every
+    CTA of the engine has a state of 18 doubles a sample, in the second launch
+    none has."""
+    rho = torch.from_numpy(inputs.density_gaussian(8, 0.2).rho).cuda()
+    K = samples(4 * 2560)
+    pr = sp.make_proj(1e-3, 1e-5, 0.5, 5)
+
+    def call(c, mode):
+        sp.sparkling_set_projection(c, mode)
+        sp.sparkling_step_batched(c, K, [0, 4 * 2560], 2560, [sp.make_grid(rho)], [1e-5], [pr])
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    items = asked(sp, lambda c: call(c, sp.PROJECTION_FP64))
+    assert items - asked(sp, lambda c: call(c, sp.PROJECTION_DEFAULT)) >= sms * 18 * 8 * 2560

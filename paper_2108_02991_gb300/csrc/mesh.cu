@@ -318,6 +318,7 @@ __global__ void gather_kernel(const float4 *__restrict__ pos, const int *__restr
 // targets a lane 85 ms (larger boxes, half the shuffles).
 
 constexpr int kCluster = 32;
+constexpr float kFar = 1e17f;
 
 // Spread the low 10 bits of v to every third bit.
 __device__ __forceinline__ unsigned int spread3(unsigned int v)
@@ -398,7 +399,9 @@ template <int W> __device__ __forceinline__ void box_union(Box &b)
 
 // The samples' positions in sorted order and the boxes of their clusters (one
 // warp a cluster).  Coordinates are multiplied by `unit`, a power of two (no
-// rounding), which puts sigma into [1/2, 1).
+// rounding), which puts sigma into [1/2, 1).  A sample that is not a number or so
+// far away that squares overflow -- the call reports it -- goes where it is near
+// to no other and outside its cluster's box: it spoils no other sample's sums.
 __global__ void sorted_clusters_kernel(const int *__restrict__ idx, const float4 *__restrict__ pos,
                                        int64_t N, int64_t n0, float unit, float4 *spos, Box *boxes)
 {
@@ -410,8 +413,9 @@ __global__ void sorted_clusters_kernel(const int *__restrict__ idx, const float4
         if (k < N) {
             float4 p = pos[idx[k]];
             p.x *= unit; p.y *= unit; p.z *= unit;
+            if (fabsf(p.x) < kFar && fabsf(p.y) < kFar && fabsf(p.z) < kFar) b.lo = b.hi = p;
+            else p = make_float4(kFar, kFar, kFar, 0.f);
             spos[k] = p;
-            b.lo = b.hi = p;
         }
         box_union<32>(b);
         if (lane == 0) boxes[c] = b;

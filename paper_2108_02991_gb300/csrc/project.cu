@@ -335,7 +335,8 @@ bool project_reg_applies(int dtype, int Ns, double alpha, double beta, double bo
                          const double *pin, int pin_index, int n_iter)
 {
     if (tol > 0.0 || n_iter > kMomentumMax || Ns > kRegMaxCtas * 2 * reg_max_threads(2)) return false;
-    if (dtype != 0) return true;
+    // radii whose squares are normal numbers (a row's square above them is, too)
+    if (dtype != 0) return alpha >= 1e-150 && beta >= 1e-150;
     // two-float form: radii and box whose squares and low parts stay normal
     constexpr double lo = 1.0 / (1ll << 40), hi = (double)(1ll << 40);
     auto radius_ok = [&](double r) { return std::isinf(r) || (r >= lo && r <= hi); };

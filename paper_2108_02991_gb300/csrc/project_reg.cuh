@@ -268,15 +268,16 @@ __device__ __forceinline__ void r_update(const VecD &z, double r, double r2, con
     const unsigned long long zb = (unsigned long long)__double_as_longlong(zz);
     const bool on = exists && zb > (unsigned long long)__double_as_longlong(r2);
     if (on) {
-        if ((unsigned int)(zb >> 32) - 0x00100000u < 0x7fe00000u) {
-            double x;
-            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(zz));
-            const double e = fma(-zz * x, x, 1.0);
-            x = fma(x * e, fma(0.375, e, 0.5), x);
-            f = fma(-r, x, 1.0);
-        } else if (zz == zz) {                 // subnormal or infinite
-            f = fma(-r, rsqrt(zz), 1.0);
-        }                                      // NaN stays in its component
+        double x;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(zz));
+        const double e = fma(-zz * x, x, 1.0);
+        x = fma(x * e, fma(0.375, e, 0.5), x);
+        f = fma(-r, x, 1.0);
+        // 1/|z| = 0 where the square overflows; NaN stays in its component (zz is
+        // not subnormal: r2 is not).  A selection, not a branch: 3 % of a short
+        // shot's chain of 37 x 129 samples.
+        const unsigned int zh = (unsigned int)(zb >> 32);
+        f = zh >= 0x7ff00000u ? (zh == 0x7ff00000u ? 1.0 : 0.0) : f;
     }
     auto row = [&](double zc, double &qc, double &yc) {
         const double qn = on ? zc * f : 0.0;

@@ -100,3 +100,15 @@ def test_infinities_are_clipped(sp, ctx, dt):
     big[70, 1], big[71, 2] = 1e18, -1e18      # beyond any dual's reach
     want = oracle.project(big.astype(np.float64), 2, 200, 0.01, 1e-4, n_iter=20)
     np.testing.assert_allclose(out, want, rtol=0, atol=1e-11 if dt == np.float64 else 2.0 ** -24)
+
+
+@pytest.mark.parametrize("Nc,Ns,at", [(1, 300, 3), (2, 900, 899), (2, 1100, 5), (300, 40, 7), (40, 1300, 640), (400, 1300, 640)])
+def test_not_a_number_reaches_the_other_ctas(sp, ctx, Nc, Ns, at):
+    """One CTA, halos, clusters: the shot's other CTAs take part, other shots not."""
+    K = np.cumsum(np.random.default_rng(Ns).normal(scale=0.002, size=(Nc, Ns, 3)), axis=1).reshape(-1, 3)
+    K[at, 2] = np.nan
+    a, b = 1.0 / (2 * Ns), 1.0 / (8 * Ns * Ns)
+    out = project(sp, ctx, K, Nc, Ns, a, b, 0.5, 40)
+    want = oracle.project(K, Nc, Ns, a, b, n_iter=40)
+    np.testing.assert_array_equal(np.isnan(out), np.isnan(want))
+    np.testing.assert_allclose(out, want, rtol=0, atol=1e-11)

@@ -687,9 +687,11 @@ def run_ours(args):
             "config": {"workload": w.desc, "N": w.N, "P": int(p0.grid.rho.size),
                        "trajectories": len(w.probs), "Ns": w.Ns, "pairs_per_step": w.pairs,
                        "n_pit": p0.proj.n_iter,
-                       "path": (("engine, one launch" if w.one_launch else "engine")
-                                if w.batched else
-                                "engine, one launch" if ktimes["engine"][1] else "kernels"),
+                       "path": (("engine, pair items in one launch" if w.one_launch else
+                                 "engine, symmetric repulsion ahead of it")
+                                + (", projection items" if args.projection == "fp64" else
+                                   ", projections after it")
+                                if w.batched or ktimes["engine"][1] else "kernels"),
                        "l2": "flushed (512 MB write) before every step", "acc": args.acc,
                        "projection": args.projection,
                        "attraction": args.attraction, "repulsion": args.repulsion,

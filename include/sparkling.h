@@ -276,13 +276,15 @@ SPARKLING_API int sparkling_project(sparkling_ctx *ctx, void *K, int K_dtype, in
  * (so eta = 1/N is a unit step on dF/dK).  The gradient is kept in FP64 in
  * the workspace; the step and the projection run in FP64 (unless the
  * context chose SPARKLING_PROJECTION_MIXED) and the result is rounded to
- * K_dtype (two-float sums for FP32 K: sparkling_set_projection).  With timing on, the device work of the call is also timed as one
- * SPARKLING_KERNEL_STEP scope.  The device work runs either as the separate
- * kernels or on the persistent engine (sparkling_step_batched with B = 1: the
- * same arithmetic, attraction and symmetric repulsion items of one launch
- * sharing the SMs, FP32 samples projected by a second launch), as
- * sparkling_set_step_path chooses; the engine applies
- * with direct sums, ACC_KAHAN32 or ACC_FP64 and a fixed n_iter.
+ * K_dtype (two-float sums for FP32 K: sparkling_set_projection).  With timing
+ * on, the device work of the call is also timed as one SPARKLING_KERNEL_STEP
+ * scope.  The device work runs either as the separate kernels or on the
+ * persistent engine (sparkling_step_batched with B = 1: attraction and symmetric
+ * repulsion items of one launch sharing the SMs, FP32 samples projected by a
+ * second launch; the same arithmetic above 11264 samples, below which the
+ * kernels sum the repulsion directed -- other FP32 roundings, ~1e-7), as
+ * sparkling_set_step_path chooses; the engine applies with direct sums,
+ * ACC_KAHAN32 or ACC_FP64 and a fixed n_iter.
  * Asynchronous on the kernels path unless converged mode is requested; the
  * engine path first waits for the stream's earlier work. */
 SPARKLING_API int sparkling_step(sparkling_ctx *ctx, void *K, int K_dtype, int64_t Nc, int64_t Ns,
@@ -398,14 +400,19 @@ SPARKLING_API int sparkling_set_autotune(sparkling_ctx *ctx, int enable);
  * the autotuner's choice.  kernel = SPARKLING_KERNEL_ATTRACTION: variant 0,
  * 1, 2 = 128, 256, 512 threads per CTA (8, 4, 2 targets per thread).
  * kernel = SPARKLING_KERNEL_REPULSION (the symmetric kernel of
- * sparkling_grad, sparkling_energy, sparkling_step and the batched step):
+ * sparkling_grad, sparkling_energy, sparkling_step and the batched step; up to
+ * 11264 samples the first three sum the repulsion directed unless a shape is
+ * pinned, which takes 8 us instead of 78 at 1024 samples and 71 instead of 88 at
+ * 11000, so a pin for the sake of one call costs the others of the context):
  * variant 0 = 256 threads per CTA (4 targets per lane), 2 sources per lane,
  * targets paired in the 64-bit registers; 1 = 256 threads, 4 sources per
  * lane, targets paired; 2 = 256 threads, 2 sources per lane, the two sources
  * paired; 3 = 128 threads per CTA (8 targets per lane), 2 sources paired
  * (the shape used where nothing is tuned or pinned, e.g. by the batched
- * step).  variant = -1 unpins (the next call of a new key tunes
- * again when the autotuner is on).  sparkling_set_autotune(ctx, -1) unpins
+ * step; unpinned, the energy takes shape 2, and below 65536 samples the number of
+ * tile pairs decides between 2 and 3).  variant = -1 unpins (the next call of a
+ * new key tunes again when the autotuner is on).  Unpinned, the pass that forms
+ * force and energy together takes attraction shape 2.  sparkling_set_autotune(ctx, -1) unpins
  * both.  Returns SPARKLING_E_INVAL for another kernel or variant. */
 SPARKLING_API int sparkling_set_shape(sparkling_ctx *ctx, int kernel, int variant);
 
@@ -510,7 +517,8 @@ SPARKLING_API int sparkling_set_attraction(sparkling_ctx *ctx, int mode);
  *     needs them (blocking; about 384 M^3 bytes of temporary device memory,
  *     M = n_cells + 2g), again when the mesh or the regularisation changes;
  *     the context then keeps about 330 M^3 bytes (spectra, FFT and charge
- *     buffers) plus 58 bytes per sample.  A sample outside the mesh gives
+ *     buffers) plus 66 bytes per sample (and 32 of the workspace).  A sample
+ *     outside the mesh gives
  *     SPARKLING_E_RANGE.  The first evaluation of a sample count sizes the
  *     buffers; later evaluations are asynchronous, so after one such call
  *     outside any stream capture they can be captured into a CUDA graph.  A

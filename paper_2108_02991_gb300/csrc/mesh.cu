@@ -308,14 +308,16 @@ __global__ void gather_kernel(const float4 *__restrict__ pos, const int *__restr
 // near one half of the group only meets that half.
 //
 // Bound: the FP32 and SFU pipes together (22 lane operations and three SFU
-// results an unordered pair; at four targets a lane ncu has them 67 and 61 %
-// busy, the warps of an SM moving through the same step in phase).  Measured
-// against the cell list before it (directed pairs, cells of rc/3, every source
-// of 49 neighbour rows tested against 64 targets): 1e7 samples, 256 cells
-// 176 -> 71 ms; 1e6 samples on spokes, 128 cells 250 -> 80 ms.  On the way, 1e7 /
-// 1e6 samples: directed with the sources culled against the boxes 124 / 152 ms,
-// symmetric pairs 133 / 90, Hilbert instead of Morton order 82 / 77 ms; with four
-// targets a lane 85 ms (larger boxes, half the shuffles).
+// results an unordered pair evaluated, of which one in 3.4 is in range at 1e7
+// samples on 256 cells and one in 1.4 at 1e6 on 128); 65536 samples on 64 cells:
+// ncu has the FMA pipe 57 % and the SFU 49 % busy, the warps of an SM moving
+// through the same step in phase.  Measured against the cell list before it
+// (directed pairs, cells of rc/3, every source of 49 neighbour rows tested against
+// 64 targets): 1e7 samples, 256 cells 176 -> 71 ms; 1e6 samples on spokes, 128
+// cells 250 -> 80 ms.  On the way, 1e7 / 1e6 samples: directed with the sources
+// culled against the boxes 124 / 152 ms, symmetric pairs 133 / 90, Hilbert instead
+// of Morton order 82 / 77 ms; with four targets a lane 85 ms (larger boxes, half
+// the shuffles).
 
 constexpr int kCluster = 32;
 constexpr float kFar = 1e17f;

@@ -13,10 +13,11 @@
 //
 // Fixed iterations run in the register form (project_reg.cuh) up to 8192
 // samples a shot.  What follows is the form with its state in memory, for
-// converged mode, longer shots, more iterations than the momentum table holds
-// and radii outside the two-float range; there FP32 samples may (an opt-in of
-// the context) iterate in FP32 on the displacement s - k and the duals
-// (project_shot_mixed), else in FP64.
+// converged mode, longer shots, more iterations than the momentum table holds,
+// radii outside the two-float range (FP64 samples: with subnormal squares) and
+// FP32 samples of a context that asked for FP64.  Outside the register form FP32
+// samples may (an opt-in of the context) iterate in FP32 on the displacement
+// s - k and the duals (project_shot_mixed), else in FP64.
 //
 // One CTA per shot (grid-stride over shots).  The 18 per-sample FP64 arrays
 // (k, s, y1, y2, q1, q2; x, y, z each, structure of arrays so that a warp

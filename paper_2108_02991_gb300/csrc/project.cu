@@ -295,9 +295,9 @@ __global__ void __launch_bounds__(reg_max_threads(M)) project_batch_kernel(const
     }
 }
 
-// Violations of the result, a thread a sample whatever the shots' length: the
-// maxima are taken over all of them, so a block reduces once and not a shot at a
-// time.
+// Violations of the result: the maxima are taken over all samples, so a block
+// reduces once.  Shots of 256 samples and more are taken block by block; of
+// shorter ones a block holds many, a thread a sample.
 template <typename KT>
 __global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
 {
@@ -308,15 +308,22 @@ __global__ void __launch_bounds__(256) violation_kernel(const ProjArgs p)
     sp.pin_index = p.pin_index; sp.n_iter = p.n_iter; sp.check_every = 0;
     sp.viol = p.viol; sp.notconv = nullptr;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    const unsigned int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
-    const int dshot = (int)(step / (unsigned int)p.Ns), dn = (int)(step % (unsigned int)p.Ns);
-    int64_t shot = first / (unsigned int)p.Ns;
-    int n = (int)(first % (unsigned int)p.Ns);
-    while (shot < p.Nc) {
-        sample_violation<KT>(static_cast<const KT *>(p.K) + 3 * shot * p.Ns, n, sp, v);
-        shot += dshot;
-        n += dn;
-        if (n >= p.Ns) { n -= p.Ns; ++shot; }
+    const KT *K = static_cast<const KT *>(p.K);
+    if (p.Ns >= (int)blockDim.x) {
+        for (int64_t shot = blockIdx.x; shot < p.Nc; shot += gridDim.x)
+            for (int n = threadIdx.x; n < p.Ns; n += blockDim.x)
+                sample_violation<KT>(K + 3 * shot * p.Ns, n, sp, v);
+    } else {
+        const unsigned int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+        const int dshot = (int)(step / (unsigned int)p.Ns), dn = (int)(step % (unsigned int)p.Ns);
+        int64_t shot = first / (unsigned int)p.Ns;
+        int n = (int)(first % (unsigned int)p.Ns);
+        while (shot < p.Nc) {
+            sample_violation<KT>(K + 3 * shot * p.Ns, n, sp, v);
+            shot += dshot;
+            n += dn;
+            if (n >= p.Ns) { n -= p.Ns; ++shot; }
+        }
     }
     reduce_violation(v, sp);
 }
@@ -477,6 +484,7 @@ cudaError_t launch_project_reg(const ProjArgs &p, int dtype, const RegShape &s, 
     const int64_t total = p.Nc * p.Ns, one = (total + 255) / 256, two = (total + 511) / 512;
     int64_t g = two < (int64_t)sms * 4 ? two : (int64_t)sms * 4;
     if (g < sms) g = one < sms ? one : sms;
+    if (p.Ns >= 256) g = p.Nc < (int64_t)sms * 8 ? p.Nc : (int64_t)sms * 8;
     if (dtype == 0) violation_kernel<float><<<(unsigned)g, 256, 0, st>>>(p);
     else violation_kernel<double><<<(unsigned)g, 256, 0, st>>>(p);
     return cudaGetLastError();

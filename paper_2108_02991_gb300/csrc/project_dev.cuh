@@ -418,8 +418,8 @@ __device__ __forceinline__ void sample_violation(const KT *Kshot, int n, const S
     }
 }
 
-// The threads' maxima, of one block, into p.viol (where they are larger: the
-// blocks' atomics meet at four words).
+// The threads' maxima, of one block, into p.viol (of many blocks, whose atomics
+// meet at four words, where they are larger).
 __device__ __forceinline__ void reduce_violation(double v[4], const ShotParams &p)
 {
     double unused = 0.0;
@@ -427,7 +427,8 @@ __device__ __forceinline__ void reduce_violation(double v[4], const ShotParams &
     if (threadIdx.x == 0)
         for (int e = 0; e < 4; ++e) {
             const unsigned long long bits = (unsigned long long)__double_as_longlong(fmax(v[e], 0.0));
-            if (bits > *(volatile unsigned long long *)&p.viol[e]) atomicMax(&p.viol[e], bits);
+            if (gridDim.x < 128 || bits > *(volatile unsigned long long *)&p.viol[e])
+                atomicMax(&p.viol[e], bits);
         }
 }
 

@@ -20,11 +20,12 @@ from __future__ import annotations
 
 import torch
 
+from . import make_grid, sparkling_energy, sparkling_energy_backward_kept, sparkling_energy_keep
+
 
 class SparklingEnergy(torch.autograd.Function):
     @staticmethod
     def forward(ctx_, K, rho, lo, hi, lib_ctx, acc, keep=True):
-        from . import make_grid, sparkling_energy, sparkling_energy_keep
         grid = make_grid(rho, lo, hi)
         A, ctx_.eps = None, -1.0
         if keep and ctx_.needs_input_grad[0]:
@@ -37,10 +38,9 @@ class SparklingEnergy(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx_, grad_out):
-        from . import make_grid, sparkling_energy_backward_kept
         K, rho, A = ctx_.saved_tensors
         grid = make_grid(rho, ctx_.lo, ctx_.hi)
-        g = grad_out.detach().to(torch.float64).contiguous()
+        g = grad_out.to(torch.float64).contiguous()        # only its values are read
         dK = sparkling_energy_backward_kept(ctx_.lib_ctx, K, grid, A, ctx_.eps, g=g, scale=1.0,
                                             acc=ctx_.acc)
         return dK, None, None, None, None, None, None

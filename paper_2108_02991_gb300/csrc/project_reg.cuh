@@ -258,6 +258,11 @@ __device__ __forceinline__ bool v_near(const VecDf &v, Df box)
 //
 // FP64: q itself is kept, Y+ = q+ + mom (q+ - q).  A warp whose rows all lie
 // inside the ball skips the factor (the FP64 pipe bounds this form).
+// Where the square overflows 1/|z| is 0, and NaN stays in its component (zz is not
+// subnormal: r2 is not).  Selections, not a branch (3 % of 37 x 129 samples): of the
+// factor with two samples a thread, of the products with one, whose chain bounds it
+// (37 x 129 293 us, selecting the factor 299; 127 x 2047 7.55 ms, factor 7.53).
+template <int M>
 __device__ __forceinline__ void r_update(const VecD &z, double r, double r2, const double2 m,
                                          bool exists, VecD &q, VecD &y)
 {
@@ -267,20 +272,22 @@ __device__ __forceinline__ void r_update(const VecD &z, double r, double r2, con
     // compares above)
     const unsigned long long zb = (unsigned long long)__double_as_longlong(zz);
     const bool on = exists && zb > (unsigned long long)__double_as_longlong(r2);
+    const unsigned int zh = (unsigned int)(zb >> 32);
     if (on) {
         double x;
         asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(zz));
         const double e = fma(-zz * x, x, 1.0);
         x = fma(x * e, fma(0.375, e, 0.5), x);
         f = fma(-r, x, 1.0);
-        // 1/|z| = 0 where the square overflows; NaN stays in its component (zz is
-        // not subnormal: r2 is not).  A selection, not a branch: 3 % of a short
-        // shot's chain of 37 x 129 samples.
-        const unsigned int zh = (unsigned int)(zb >> 32);
-        f = zh >= 0x7ff00000u ? (zh == 0x7ff00000u ? 1.0 : 0.0) : f;
+        if (M > 1) f = zh >= 0x7ff00000u ? (zh == 0x7ff00000u ? 1.0 : 0.0) : f;
     }
+    const bool odd = M == 1 && on && zh >= 0x7ff00000u;
     auto row = [&](double zc, double &qc, double &yc) {
-        const double qn = on ? zc * f : 0.0;
+        double qn = on ? zc * f : 0.0;
+        if (M == 1) {
+            const bool nan = (__double2hiint(zc) & 0x7fffffff) >= 0x7ff00000;
+            qn = odd ? (zh == 0x7ff00000u || nan ? zc : 0.0) : qn;
+        }
         yc = fma(m.x, qn - qc, qn);
         qc = qn;
     };
@@ -292,6 +299,7 @@ __device__ __forceinline__ void r_update(const VecD &z, double r, double r2, con
 // Two floats: W = mom q is kept, Y+ = ((1 + mom) f) z - W and W+ = (mom+ f) z
 // (q+ itself in the last iteration).  No branch: both rows of a sample and
 // their long dependent chains run side by side.
+template <int M>
 __device__ __forceinline__ void r_update(const VecDf &z, Df r, float r2, const float4 m, bool exists,
                                          VecDf &w, VecDf &y)
 {
@@ -469,8 +477,8 @@ __device__ __forceinline__ void project_registers(const RegShot &p, const Moment
         for (int j = 0; j < M; ++j) {
             const V z1 = v_add(y1[j], d[j]);
             const V z2 = v_add(y2[j], v_sub_raw(j + 1 < M ? d[j + 1 < M ? j + 1 : 0] : dr, d[j]));
-            r_update(z1, alpha, a2, mo, m0 + j < p.Ns - 1, w1[j], y1[j]);
-            r_update(z2, beta, b2, mo, m0 + j < p.Ns - 2, w2[j], y2[j]);
+            r_update<M>(z1, alpha, a2, mo, m0 + j < p.Ns - 1, w1[j], y1[j]);
+            r_update<M>(z2, beta, b2, mo, m0 + j < p.Ns - 2, w2[j], y2[j]);
             if (final) {          // the output is s(q), not s(Y)
                 y1[j] = w1[j];
                 y2[j] = w2[j];
